@@ -26,6 +26,7 @@
 #include "lola_run_tc.cuh"
 #include "lola_team_tc.cuh"
 #include "lola_unit_f32.cuh"
+#include "lola_step_f32.cuh"
 
 using namespace lola;
 
@@ -244,6 +245,7 @@ struct lola_state {
   int team_fit[9] = {};                // prefill kernel with attention and scoring blocks: clusters of 2 .. 8 that are resident at once
   int run_blocks = 0;                  // bf16 layers: blocks per unit of the one-kernel prefill run (0: not used)
   int unit_blocks = 0;                 // fp32 layers: blocks per unit of the one-kernel step (0: its shape does not fit)
+  int step_blocks = 0;                 // ... and of the generation step with F = 64 (0: not used)
   CUtensorMap tm_gk, tm_gv, tm_wk, tm_wv;
   lola_call_info info = {};            // what the last prefill / decode call enqueued
   bool profiling = false;
@@ -409,6 +411,16 @@ int launch_update_chain(lola_state* st, const Call& c, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? LOLA_OK : LOLA_ERR_CUDA;
 }
 
+// fp32 layers with F = 64: a generation step.
+template <int DPL>
+int launch_unit_step(lola_state* st, const Call& c, cudaStream_t s) {
+  const Layer& L = st->L;
+  const int K = st->step_blocks, grid = L.B * L.Hkv * K;
+  LaunchScope scope(st, LOLA_KERNEL_DECODE, s, LOLA_PATH_UNIT_RUN, grid);
+  const cudaError_t le = launch_pdl_cluster(k_unit_step<DPL>, K, dim3(grid), dim3(kStepThreads), sizeof(StepSmem<DPL>), s, L, c);
+  return le == cudaSuccess && cudaGetLastError() == cudaSuccess ? LOLA_OK : LOLA_ERR_CUDA;
+}
+
 // fp32 layers: a run of prefill chunks, or one generation step, as one kernel.
 template <int DPL>
 int launch_unit_run(lola_state* st, const Call& c, int n_chunks, bool decode, cudaStream_t s) {
@@ -566,6 +578,7 @@ int launch_decode_fused(lola_state* st, const Call& c, cudaStream_t s) {
 
 template <typename T, int DPL>
 int run_decode(lola_state* st, Call c, cudaStream_t s) {
+  if (st->step_blocks > 0 && !st->force_chain) return launch_unit_step<DPL>(st, c, s);
   if (st->unit_blocks > 0 && !st->force_chain) return launch_unit_run<DPL>(st, c, 1, true, s);
   // the whole step is one kernel, with full caches (UPD_SELECT) and while they fill (UPD_NONE, UPD_APPEND)
   const bool ablation = (st->cfg.flags & (LOLA_FLAG_QUERY_NO_LINEAR | LOLA_FLAG_QUERY_NO_SPARSE)) != 0;
@@ -662,6 +675,11 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
         (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_run<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)
                               : cudaFuncSetAttribute(k_unit_run<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) == cudaSuccess)
       st->unit_blocks = K;
+    const bool ablation = (cfg->flags & (LOLA_FLAG_QUERY_NO_LINEAR | LOLA_FLAG_QUERY_NO_SPARSE)) != 0;
+    if (cfg->feat_half == 64 && cfg->sparse >= 1 && cfg->window >= 1 && L.g <= kStepQ && !ablation &&
+        (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_step<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem<4>))
+                              : cudaFuncSetAttribute(k_unit_step<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StepSmem<2>))) == cudaSuccess)
+      st->step_blocks = K;
   }
   if (rc == LOLA_OK && st->tensor_path) {
     cudaError_t e = cfg->head_dim == 128

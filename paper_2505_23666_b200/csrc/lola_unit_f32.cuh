@@ -1,4 +1,5 @@
-// The whole step of an fp32 layer - a run of prefill chunks, or one generation step - as ONE kernel: a cluster of K
+// The whole step of an fp32 layer - a run of prefill chunks, or one generation step of the shapes that k_unit_step does not
+// serve (F other than 64, no window or no sparse cache, query restrictions, more than 8 query heads) - as ONE kernel: a cluster of K
 // thread blocks carries one (batch row, KV head) unit through the run, all arithmetic in fp32 on the CUDA cores.
 //
 // What bounds it: latency.  A chunk of the tiny fp32 layer (64 tokens, 256 keys, d = 64) is 6 MFMA per unit; as a
