@@ -42,15 +42,15 @@ constexpr int kRunMaxN = 64;         // tokens per chunk (and folds: one batch o
 
 template <int NQ>
 struct RunMisc {
-  unsigned key[run_max_e(NQ)];       // score bits of E
+  alignas(16) unsigned key[run_max_e(NQ)];   // score bits of E
   short cand[run_max_e(NQ)];         // scratch of the selection
   unsigned char mark[run_max_e(NQ)];
   short fold[kRunMaxN];              // E indices of the folded pairs
   short dst[kRunMaxN];               // per leaving pair: slot it takes, or -1
-  short freed[kRunMaxN];
   SelectScratch sel;
   float s[128];                      // the normaliser state, fp32 (the same in every block)
   float ssp[128];
+  float2 phx[2][128];                // fold: maximum and sum of a thread's 32 features
   union {
     float redm[4][64];               // per row quadrant: column maxima of a tile
     float l_s[4][64];                // after the last tile: sums of the weights
@@ -657,8 +657,25 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
         if (tid == 0) tc::mbar_expect_tx(BAR(R_SCORES), (uint32_t)nE * 4u);
         WAIT(R_SCORES, ph_sc & 1);                     // the scores of all blocks are here
         ++ph_sc;
+        constexpr int PPR = d / 4;                     // 16-byte pieces of a pair: key, then value
+        constexpr int NP = kUp2Batch * PPR / 256;
+        uint4 val[NP];                                 // the folded pairs, on their way as soon as they are known
+        const int isv = (tid % PPR) / (PPR / 2), ch = tid % (PPR / 2);
         select_lists<256>(X.key, [&](int e) { return e < cg ? __ldcg(L.gpos + (size_t)unit * lam + e) : c.r_pos0 + (e - cg); }, X.cand, X.mark, nE, nF, cg,
-                          X.fold, X.freed, X.dst, X.sel, tid, sync, [] {});
+                          X.fold, X.sel, tid, sync, [&](int i, int to) { X.dst[i] = (short)to; }, [&] {
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            const int row = tid / PPR + q * (256 / PPR);
+            val[q] = make_uint4(0, 0, 0, 0);
+            if (row < nF) {
+              const int e = X.fold[row];
+              int slot = ring0 + e - cg;
+              if (slot >= eta) slot -= eta;
+              const T* base = e < cg ? (const T*)(isv ? L.gv : L.gk) + ((size_t)unit * lam + e) * d : (const T*)(isv ? L.wv : L.wk) + ((size_t)unit * eta + slot) * d;
+              val[q] = __ldcg(reinterpret_cast<const uint4*>(base + ch * 8));
+            }
+          }
+        });
         if (rank == 0 && tid == 0 && ok) {
           L.thr[(size_t)unit * 2 + 0] = __uint_as_float(X.sel.min_keep);
           L.thr[(size_t)unit * 2 + 1] = __uint_as_float(X.sel.max_fold);
@@ -673,22 +690,6 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           for (int j = 0; j < 8; ++j) hv[j] = Hg[(size_t)((it >> dKs) * 8 + j) * d + c0 + (it & (dK - 1))];
         };
         {
-          constexpr int PPR = d / 4;                   // 16-byte pieces of a pair: key, then value
-          constexpr int NP = kUp2Batch * PPR / 256;
-          uint4 val[NP];
-          const int isv = (tid % PPR) / (PPR / 2), ch = tid % (PPR / 2);
-#pragma unroll
-          for (int q = 0; q < NP; ++q) {
-            const int row = tid / PPR + q * (256 / PPR);
-            val[q] = make_uint4(0, 0, 0, 0);
-            if (row < nF) {
-              const int e = X.fold[row];
-              int slot = ring0 + e - cg;
-              if (slot >= eta) slot -= eta;
-              const T* base = e < cg ? (const T*)(isv ? L.gv : L.gk) + ((size_t)unit * lam + e) * d : (const T*)(isv ? L.wv : L.wk) + ((size_t)unit * eta + slot) * d;
-              val[q] = __ldcg(reinterpret_cast<const uint4*>(base + ch * 8));
-            }
-          }
           tc::named_bar_sync(3, 512);                  // the attention group is done with the stages, which the tiles lie over
 #pragma unroll
           for (int q = 0; q < NP; ++q) {
@@ -719,28 +720,38 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           ++ph_s;
           tc::fence_after_sync();
           {
-            // rows 0-63 the pairs' first parts, 64-127 the second ones; the third ones, if taken, in the rows of the value
-            // tile that hold no pair
+            // lanes t and t + 64 hold the same pair and take 32 features of their half each: first parts into rows 0-63, second
+            // ones into 64-127; the third ones, if taken, into the rows of the value tile that hold no pair
             const bool ek = L.phi_kind == 1;
-            uint32_t u[64];
-            uint64_t x2[32];
-            tc::tmem_ld64u(tm_u + lane_addr, u);
-            const uint64_t inv2 = tc::phi_half_f32(u, hf != 0, ek, x2);
+            const int pr = t & 63, qh = t >> 6;
+            uint32_t u[32];
+            uint64_t x2[16];
+            float m, sum, f = 1.0f;
+            tc::tmem_ld32u(tm_u + lane_addr + qh * 32, u);
+            tc::phi_quarter_f32(u, hf != 0, ek, x2, m, sum);
+            if (!ek) {
+              X.phx[hf][t] = make_float2(m, sum);
+              tc::named_bar_sync(6 + hf * 2 + (wq & 1), 64);   // the two warps that share these pairs
+              const float2 o = X.phx[hf][t ^ 64];
+              const float mm = fmaxf(m, o.x), a = tc::fast_exp2(m - mm);
+              f = a / fmaf(sum, a, o.y * tc::fast_exp2(o.x - mm));
+            }
+            const uint64_t f2 = tc::pack_f2(f, f);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              uint32_t pk[4];
+            for (int q = 0; q < 4; ++q) {
+              uint32_t p1[4], p2[4], p3[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                if (!ek) x2[q * 4 + e] = tc::mul2(x2[q * 4 + e], inv2);
-                pk[e] = tc::phi_part(x2[q * 4 + e], t >= 64);
+                float a, b;
+                tc::unpack_f2(tc::mul2(x2[q * 4 + e], f2), a, b);
+                p1[e] = tc::next_part(a, b);
+                p2[e] = tc::next_part(a, b);
+                if (THREE) p3[e] = tc::next_part(a, b);
               }
-              *reinterpret_cast<uint4*>(sm + S::fold_k + hf * 16384 + tc::sw128_off(t, q)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            }
-            if (THREE && three && t >= 64) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q)
-                *reinterpret_cast<uint4*>(sm + S::fold_v + hf * 16384 + tc::sw128_off(t, q)) =
-                    make_uint4(tc::phi_third(x2[q * 4]), tc::phi_third(x2[q * 4 + 1]), tc::phi_third(x2[q * 4 + 2]), tc::phi_third(x2[q * 4 + 3]));
+              const uint32_t off = tc::sw128_off(pr, qh * 4 + q), dst = S::fold_k + hf * 16384;
+              *reinterpret_cast<uint4*>(sm + dst + off) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+              *reinterpret_cast<uint4*>(sm + dst + 8192 + off) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
+              if (THREE && three) *reinterpret_cast<uint4*>(sm + S::fold_v + hf * 16384 + 8192 + off) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
             }
           }
           tc::fence_async_smem();

@@ -38,12 +38,11 @@ struct TeamAttMisc {
   int abort_word;
 };
 struct TeamScoreMisc {
-  unsigned key[kTeamMaxE];           // score bits of E
+  alignas(16) unsigned key[kTeamMaxE];   // score bits of E
   short cand[kTeamMaxE];             // scratch of the selection
   unsigned char mark[kTeamMaxE];
   short fold[kTeamMaxN];             // E indices of the folded pairs
   short dst[kTeamMaxN];              // per leaving pair: slot it takes, or -1
-  short freed[kTeamMaxN];
   SelectScratch sel;
   alignas(16) float s[128];          // the normaliser state, fp32 (the same in every scoring block)
   float ssp[2][128];
@@ -698,19 +697,21 @@ k_prefill_team(Layer L, Call c, int n_chunks, const __grid_constant__ TeamMaps M
           }
         };
         select_lists<512>(X.key, [&](int e) { return e < cg ? __ldcg(L.gpos + (size_t)unit * lam + e) : c.r_pos0 + (e - cg); }, X.cand, X.mark, nE, nF, cg,
-                          X.fold, X.freed, X.dst, X.sel, tid, sync_all, [&] {
+                          X.fold, X.sel, tid, sync_all,
+                          [&](int i, int to) {
+                            X.dst[i] = (short)to;
+                            if (sr == 0 && ok) L.move_dst[(size_t)unit * L.cmax + i] = to;   // (read by the attention blocks)
+                          },
+                          [&] {
                             // (both groups are through with their tiles: the buffers may be written)
                             gather(0);
 #pragma unroll 1
                             for (int i = tid; i < dK * 32; i += 512)   // this block's columns of H
                               tc::cp_async16(sbase + hrow((i ^ ((i >> (dKs - 2)) & hm)) * 16), Hg + (size_t)(i >> (dKs - 2)) * d + c0 + (i & (dK / 4 - 1)) * 4);
                           });
-        if (sr == 0 && ok) {
-          if (tid == 0) {
-            L.thr[(size_t)unit * 2 + 0] = __uint_as_float(X.sel.min_keep);
-            L.thr[(size_t)unit * 2 + 1] = __uint_as_float(X.sel.max_fold);
-          }
-          for (int i = tid; i < c.r; i += 512) L.move_dst[(size_t)unit * L.cmax + i] = X.dst[i];   // (read by the attention blocks)
+        if (sr == 0 && tid == 0 && ok) {
+          L.thr[(size_t)unit * 2 + 0] = __uint_as_float(X.sel.min_keep);
+          L.thr[(size_t)unit * 2 + 1] = __uint_as_float(X.sel.max_fold);
         }
         // ---- Eq. 13: dH = phi(K_S)^T [V_S | 1], 64 pairs at a time, phi in two or three bf16 parts against the same values
         const bool three = LONG && fold_in_three(c);

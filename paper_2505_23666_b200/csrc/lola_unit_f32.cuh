@@ -39,7 +39,7 @@ struct UnitLayout {            // shared memory of k_unit_run, offsets in floats
   int fp, dp;                  // F and D rounded up to a multiple of 4 (zero padding)
   int jn, jsh;                 // rows of H a block folds, and the power of two that covers them
   int phi_ld;
-  int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, freed, dst, sel, src, total;
+  int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, dst, sel, src, total;
 };
 
 LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
@@ -79,7 +79,6 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
   Y.cand = take(nE);
   Y.mark = take((nE + 3) / 4);
   Y.fold = take(L.cmax);
-  Y.freed = take(L.cmax);
   Y.dst = take(L.cmax);
   Y.sel = take((int)(sizeof(SelectScratch) + 3) / 4);
   Y.src = take(kUnSrcFloats);
@@ -367,7 +366,7 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
   float *Ws = sm + Y.W, *Hs = sm + Y.H, *ss = sm + Y.s, *phi = sm + Y.phi, *xs = sm + Y.xs, *den = sm + Y.den, *vf = sm + Y.vf, *pf = sm + Y.pf;
   unsigned* key = reinterpret_cast<unsigned*>(sm + Y.key);
   int *pos = reinterpret_cast<int*>(sm + Y.pos), *cand = reinterpret_cast<int*>(sm + Y.cand), *fold = reinterpret_cast<int*>(sm + Y.fold),
-      *freed = reinterpret_cast<int*>(sm + Y.freed), *dst = reinterpret_cast<int*>(sm + Y.dst);
+      *dst = reinterpret_cast<int*>(sm + Y.dst);
   unsigned char* mark = reinterpret_cast<unsigned char*>(sm + Y.mark);
   SelectScratch& S = *reinterpret_cast<SelectScratch*>(sm + Y.sel);
   UnitSrc& U = *reinterpret_cast<UnitSrc*>(sm + Y.src);
@@ -568,7 +567,8 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
       for (int i = tid; i < c.r; i += kUnThreads) pos[cg + i] = c.r_pos0 + i;
       __syncthreads();
       select_lists<kUnThreads>(key, [&](int e) { return pos[e]; }, cand, mark, nE, nF, cg,
-                               fold, freed, dst, S, tid, [] { __syncthreads(); }, [] {});
+                               fold, S, tid, [] { __syncthreads(); }, [&](int i, int to) { dst[i] = to; }, [] {});
+      __syncthreads();
       if (rank == 0 && tid == 0) {
         L.thr[(size_t)unit * 2 + 0] = __uint_as_float(S.min_keep);
         L.thr[(size_t)unit * 2 + 1] = __uint_as_float(S.max_fold);

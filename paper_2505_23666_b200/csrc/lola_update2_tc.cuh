@@ -41,13 +41,11 @@ struct Update2Smem {
 
 // shared memory of the selection
 struct SelectMisc {
-  unsigned key[kUp2MaxE];           // score bits
+  alignas(16) unsigned key[kUp2MaxE];   // score bits
   int pos[kUp2MaxE];                // positions
   int cand[kUp2MaxE];
   unsigned char mark[kUp2MaxE];     // 1: the pair folds
   int fold_e[kUp2MaxFold];          // E indices of the folded pairs, ascending
-  int free_slot[kUp2MaxFold];
-  int dst_of[kUp2MaxFold];          // per leaving pair: the slot it takes, or -1
   SelectScratch scratch;
 };
 
@@ -105,10 +103,9 @@ __device__ __forceinline__ void select_body(const Layer& L, const Call& c, uint8
   }
   __syncthreads();
   select_lists<kUp2Threads>(X.key, [&](int e) { return X.pos[e]; }, X.cand, X.mark, nE, nF, cg,
-                            X.fold_e, X.free_slot, X.dst_of, X.scratch, tid, [] { __syncthreads(); }, [] {});
+                            X.fold_e, X.scratch, tid, [] { __syncthreads(); }, [&](int i, int to) { L.move_dst[lo + i] = to; }, [] {});
   // the lists leave through the state's work-list arrays
   for (int i = tid; i < nF; i += kUp2Threads) L.fold_idx[lo + i] = X.fold_e[i];
-  for (int i = tid; i < c.r; i += kUp2Threads) L.move_dst[lo + i] = X.dst_of[i];
   if (tid == 0) {
     L.thr[(size_t)unit * 2 + 0] = __uint_as_float(X.scratch.min_keep);
     L.thr[(size_t)unit * 2 + 1] = __uint_as_float(X.scratch.max_fold);
