@@ -194,6 +194,19 @@ bool make_rows_map(CUtensorMap* tm, void* base, size_t units, size_t rows, size_
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The sparse cache [units][rows][d]: blocks as above and whole tiles.
+bool make_slot_maps(tc::SlotMaps* m, void* base, size_t units, size_t rows, size_t d) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn || rows == 0) return false;
+  cuuint64_t dims[4] = {64, rows, d / 64, units};
+  cuuint64_t strides[3] = {d * 2, 128, rows * d * 2};
+  cuuint32_t box[4] = {64, 128, (cuuint32_t)(d / 64), 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return make_rows_map(&m->block, base, units, rows, d, 64) &&
+         fn(&m->tile, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // bf16 tensor [chunks][B][n][heads][d] of a run viewed as rank 5; boxes of 64 columns x 1 head x box_tokens tokens.
 bool make_run_map(CUtensorMap* tm, const void* base, size_t chunks, size_t B, size_t n, size_t heads, size_t d, unsigned box_tokens) {
   EncodeTiledFn fn = encode_tiled_fn();
@@ -246,7 +259,8 @@ struct lola_state {
   int run_blocks = 0;                  // bf16 layers: blocks per unit of the one-kernel prefill run (0: not used)
   int unit_blocks = 0;                 // fp32 layers: blocks per unit of the one-kernel step (0: its shape does not fit)
   int step_blocks = 0;                 // ... and of the generation step with F = 64 (0: not used)
-  CUtensorMap tm_gk, tm_gv, tm_wk, tm_wv;
+  tc::SlotMaps tm_gk, tm_gv;
+  CUtensorMap tm_wk, tm_wv;
   lola_call_info info = {};            // what the last prefill / decode call enqueued
   bool profiling = false;
   std::vector<ProfRecord> records;     // events in use since the last lola_profile_read
@@ -693,8 +707,8 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
   }
   if (rc == LOLA_OK && st->tensor_path && cfg->sparse >= 1 && cfg->window >= 1) {
     const size_t U = (size_t)cfg->batch * cfg->n_kv_heads;
-    st->have_maps = make_rows_map(&st->tm_gk, L.gk, U, cfg->sparse, cfg->head_dim, 64) &&
-                    make_rows_map(&st->tm_gv, L.gv, U, cfg->sparse, cfg->head_dim, 64) &&
+    st->have_maps = make_slot_maps(&st->tm_gk, L.gk, U, cfg->sparse, cfg->head_dim) &&
+                    make_slot_maps(&st->tm_gv, L.gv, U, cfg->sparse, cfg->head_dim) &&
                     make_rows_map(&st->tm_wk, L.wk, U, cfg->window, cfg->head_dim, 64) &&
                     make_rows_map(&st->tm_wv, L.wv, U, cfg->window, cfg->head_dim, 64);
     if (!(cfg->head_dim == 128 ? set_tc_attrs<4>() : set_tc_attrs<2>())) st->have_maps = false;   // the older kernel chain serves every shape

@@ -57,7 +57,7 @@ enum { A2_QFULL = 0, A2_KFULL = 1, A2_VFULL = 3, A2_KEMPTY = 5, A2_VEMPTY = 7, A
 // LONG: chunks of more than kLagMaxN tokens
 template <int DPL, bool LONG>
 __global__ void __launch_bounds__(kAt2Threads, 1)
-k_attend2_tc(Layer L, Call c, const __grid_constant__ CUtensorMap tm_gk, const __grid_constant__ CUtensorMap tm_gv,
+k_attend2_tc(Layer L, Call c, const __grid_constant__ tc::SlotMaps tm_gk, const __grid_constant__ tc::SlotMaps tm_gv,
              const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv,
              const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ck,
              const __grid_constant__ CUtensorMap tm_cv, const __grid_constant__ CUtensorMap tm_out, const uint4* wt_image,
@@ -160,10 +160,17 @@ k_attend2_tc(Layer L, Call c, const __grid_constant__ CUtensorMap tm_gk, const _
 #pragma unroll
     for (int cb = 0; cb < kblk; ++cb) {
       const uint32_t dd = dst + (uint32_t)cb * 16384u;
-      if (blk < nGB) tc::tma_load_3d(dd, is_v ? &tm_gv : &tm_gk, cb * 64, blk * 64, unit, bar);
+      if (blk < nGB) tc::tma_load_3d(dd, is_v ? &tm_gv.block : &tm_gk.block, cb * 64, blk * 64, unit, bar);
       else if (blk < nGB + nRB) tc::tma_load_3d(dd, is_v ? &tm_wv : &tm_wk, cb * 64, (blk - nGB) * 64, unit, bar);
       else tc::tma_load_4d(dd, is_v ? &tm_cv : &tm_ck, cb * 64, h, (blk - nGB - nRB) * 64, b, bar);   // (beyond the chunk: zeros)
     }
+  };
+
+  auto issue_tile = [&](uint32_t dst, int kt, bool is_v, uint32_t bar) {
+    tc::mbar_expect_tx(bar, (uint32_t)kblk * 16384u);
+    if (2 * kt + 1 < nGB) { tc::tma_load_slots(dst, is_v ? &tm_gv : &tm_gk, kt, unit, bar); return; }
+    issue_block(dst, 2 * kt, is_v, bar);
+    issue_block(dst + 8192u, 2 * kt + 1, is_v, bar);
   };
 
   if (warp == 17) {
@@ -177,13 +184,9 @@ k_attend2_tc(Layer L, Call c, const __grid_constant__ CUtensorMap tm_gk, const _
         const uint32_t stage = sbase + S::stage0 + (uint32_t)st * S::stage_bytes;
         if (st == 1) ok = WAIT(A2_KEMPTY + 1, (kt >> 1) & 1) && ok;   // (its first completion is the read of W^T)
         else if (kt >= 2) ok = WAIT(A2_KEMPTY + 0, ((kt >> 1) - 1) & 1) && ok;
-        tc::mbar_expect_tx(BAR(A2_KFULL + st), (uint32_t)kblk * 16384u);
-        issue_block(stage + S::st_k, 2 * kt, false, BAR(A2_KFULL + st));
-        issue_block(stage + S::st_k + 8192u, 2 * kt + 1, false, BAR(A2_KFULL + st));
+        issue_tile(stage + S::st_k, kt, false, BAR(A2_KFULL + st));
         if (kt >= 2) ok = WAIT(A2_VEMPTY + st, ((kt >> 1) - 1) & 1) && ok;
-        tc::mbar_expect_tx(BAR(A2_VFULL + st), (uint32_t)kblk * 16384u);
-        issue_block(stage + S::st_v, 2 * kt, true, BAR(A2_VFULL + st));
-        issue_block(stage + S::st_v + 8192u, 2 * kt + 1, true, BAR(A2_VFULL + st));
+        issue_tile(stage + S::st_v, kt, true, BAR(A2_VFULL + st));
       }
       if (!ok) atomicOr(L.status, 64);
     }

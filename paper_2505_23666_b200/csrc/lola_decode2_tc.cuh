@@ -124,15 +124,19 @@ static_assert(sizeof(Decode2Misc) <= 28672, "misc region too small");
 // Loads of one tile: two half tiles of 64 rows; a half tile is a block of sparse-cache slots, a block
 // of ring slots, or nothing (a box that lies entirely outside the ring tensor reads as zeros).
 template <int DPL>
-__device__ __forceinline__ void decode_issue_tile(uint32_t dst, const CUtensorMap* tm_g, const CUtensorMap* tm_w, int tile,
+__device__ __forceinline__ void decode_issue_tile(uint32_t dst, const tc::SlotMaps* tm_g, const CUtensorMap* tm_w, int tile,
                                                   int nGB, int nRB, int unit, uint32_t bar) {
   constexpr int kblk = DPL / 2;
   tc::mbar_expect_tx(bar, (uint32_t)kblk * 16384u);
+  if (tile * 2 + 1 < nGB) {
+    tc::tma_load_slots(dst, tm_g, tile, unit, bar);
+    return;
+  }
 #pragma unroll
   for (int hb = 0; hb < 2; ++hb) {
     const int blk = tile * 2 + hb;
     const bool from_g = blk < nGB;
-    const CUtensorMap* tm = from_g ? tm_g : tm_w;
+    const CUtensorMap* tm = from_g ? &tm_g->block : tm_w;
     const int row = from_g ? blk * 64 : min(blk - nGB, nRB) * 64;
 #pragma unroll
     for (int cb = 0; cb < kblk; ++cb)
@@ -143,7 +147,7 @@ __device__ __forceinline__ void decode_issue_tile(uint32_t dst, const CUtensorMa
 // The tile loader as a real function: the issuing threads reach it from many places, and every inlined copy
 // would add to an instruction footprint that four different roles already share.
 template <int DPL>
-__device__ __noinline__ void decode2_issue_tile(uint32_t dst, const CUtensorMap* tm_g, const CUtensorMap* tm_w, int tile, int nGB, int nRB,
+__device__ __noinline__ void decode2_issue_tile(uint32_t dst, const tc::SlotMaps* tm_g, const CUtensorMap* tm_w, int tile, int nGB, int nRB,
                                                 int unit, uint32_t bar) {
   decode_issue_tile<DPL>(dst, tm_g, tm_w, tile, nGB, nRB, unit, bar);
 }
@@ -239,7 +243,7 @@ __device__ __noinline__ void decode_redo_rows(Decode2Misc& X, const RedoRows& R,
 // ahead: the SMs' number; the unit that many further on is likely the next one of this SM.
 template <int DPL, int QR, bool WIDE, bool SPLIT>
 __global__ void __launch_bounds__(kDec2Threads, 1)
-k_decode2_tc(Layer L, Call c, const __grid_constant__ CUtensorMap tm_gk, const __grid_constant__ CUtensorMap tm_gv,
+k_decode2_tc(Layer L, Call c, const __grid_constant__ tc::SlotMaps tm_gk, const __grid_constant__ tc::SlotMaps tm_gv,
              const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv, const uint4* wt_image, int ahead) {
   using S = DecodeSmem<DPL>;
   constexpr int d = DPL * 32;

@@ -59,7 +59,7 @@ struct RunMisc {
   float lden[2][64];                 // phi(q) . s, the two halves of the features
   float inv[64];
   int grow[3][2];
-  uint64_t bars[20];
+  uint64_t bars[23];
   uint32_t tmem_slot;
   int abort_word;
 };
@@ -119,11 +119,14 @@ __device__ __forceinline__ float cols_reduce16(const float (&v)[16], int lane) {
   return comb(a[0], __shfl_xor_sync(0xffffffffu, a[0], 1));
 }
 
-struct RunMaps { CUtensorMap gk, gv, wk, wv, q, k, v; };
+struct RunMaps {
+  tc::SlotMaps gk, gv;
+  CUtensorMap wk, wv, q, k, v;
+};
 
 // barriers
-enum { R_KFULL = 0, R_VFULL = 2, R_KEMPTY = 4, R_VEMPTY = 6, R_ZFULL = 8, R_ZFREE = 10, R_PT = 12, R_O = 13, R_OFREE = 14, R_QFULL = 15,
-       R_UQ = 16, R_PHIQ = 17, R_S = 18, R_SCORES = 19 };
+enum { R_KFULL = 0, R_VFULL = 2, R_KEMPTY = 4, R_VEMPTY = 6, R_ZFULL = 8, R_ZFREE = 10, R_PT = 12, R_O = 14, R_LIN = 16, R_OFREE = 17, R_QFULL = 18,
+       R_UQ = 19, R_PHIQ = 20, R_S = 21, R_SCORES = 22, R_N = 23 };
 
 // THREE: a kernel for runs with chunks whose fold takes phi in three parts (fold_in_three; its code costs the others up to 1 us a
 // chunk)
@@ -156,6 +159,9 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
   const float sl2 = L.scale * kLog2e;
   const int ntb = (n + 31) / 32, items = g * ntb;
   constexpr int IP = NQ / 32;                         // items of a block: rank * IP ..
+  // Buffers of the weights operand.  32 queries fill half of its 128-byte rows, so tiles take turns in the two halves and the
+  // weights of a tile are made while the product of the one before runs
+  constexpr uint32_t NB = NQ == 32 ? 2 : 1;
   const int it0 = rank * IP;
   float* scu = L.score + (size_t)unit * (lam + L.cmax);
   float* Hg = L.H + (size_t)unit * D * d;
@@ -163,8 +169,8 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
   if (tid == 0) {
     X.abort_word = 0;
     for (int i = 0; i < 6; ++i) X.grow[i / 2][i & 1] = 0;
-    for (int i = 0; i < 20; ++i)
-      tc::mbar_init(BAR(i), (i >= R_KEMPTY && i < R_ZFULL) ? 2u : (i == R_ZFREE || i == R_ZFREE + 1 || i == R_PT || i == R_OFREE) ? 256u
+    for (int i = 0; i < R_N; ++i)
+      tc::mbar_init(BAR(i), (i >= R_KEMPTY && i < R_ZFULL) ? 2u : (i == R_ZFREE || i == R_ZFREE + 1 || i == R_PT || i == R_PT + 1 || i == R_OFREE) ? 256u
                             : i == R_PHIQ ? (uint32_t)NQ * 2u : 1u);
     tc::mbar_init_fence();
     tc::grid_dep_launch_dependents();
@@ -212,7 +218,6 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
   auto stage_k = [&](uint32_t i) { return S::stage0 + (i & 1) * S::stage_bytes; };
   auto stage_v = [&](uint32_t i) { return S::stage0 + (i & 1) * S::stage_bytes + S::st_v; };
   uint32_t seq0 = 0;                                  // tiles streamed before this chunk
-  uint32_t ev = 0;                                    // attention group: O^T products waited for
   uint32_t ph_s = 0, ph_sc = 0;                       // score group: phases of R_S, R_SCORES
   uint32_t nit = 0;                                   // attention group: tiles so far
   int n_seen = c.n_seen;
@@ -232,7 +237,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
 
     if (warp == 16) {
       // =============================== key and value tiles ===============================
-      if (lane == 0) {
+      if (tc::elect_one()) {
 #pragma unroll 1
         for (TileOrder o(rank, K, n_score, n_tiles); o.own || !o.done(); o.next(), ++seq) {
             const uint32_t st = seq & 1, par = ((seq >> 1) & 1) ^ 1;
@@ -244,13 +249,17 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
               if (!ok) break;
               const uint32_t dst = sbase + (isv ? stage_v(seq) : stage_k(seq)), bar = BAR((isv ? R_VFULL : R_KFULL) + st);
               tc::mbar_expect_tx(bar, (uint32_t)kblk * 16384u);
+              if (o.t * 2 + 1 < nGB) {
+                tc::tma_load_slots(dst, isv ? &M.gv : &M.gk, o.t, unit, bar);
+                continue;
+              }
 #pragma unroll 1
               for (int hb = 0; hb < 2; ++hb) {
                 const int blk = o.t * 2 + hb;
 #pragma unroll
                 for (int cb = 0; cb < kblk; ++cb) {
                   const uint32_t dd = dst + (uint32_t)cb * 16384u + (uint32_t)hb * 8192u;
-                  if (blk < nGB) tc::tma_load_3d(dd, isv ? &M.gv : &M.gk, cb * 64, blk * 64, unit, bar);
+                  if (blk < nGB) tc::tma_load_3d(dd, isv ? &M.gv.block : &M.gk.block, cb * 64, blk * 64, unit, bar);
                   else if (blk < nGB + nRB) tc::tma_load_3d(dd, isv ? &M.wv : &M.wk, cb * 64, (blk - nGB) * 64, unit, bar);
                   else tc::tma_load_5d(dd, isv ? &M.v : &M.k, cb * 64, h, (blk - nGB - nRB) * 64, b, chunk, bar);   // (beyond the chunk: zeros)
                 }
@@ -261,7 +270,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
       __syncwarp();
     } else if (warp == 17) {
       // =============================== queries, Z = K Q^T ===============================
-      if (lane == 0) {
+      if (tc::elect_one()) {
         const uint64_t dq = tc::make_desc_sw128(sbase + S::q, 16, 1024), dw = tc::make_desc_sw128(sbase + S::wt, 16, 1024);
         const uint32_t idz = tc::make_idesc_bf16(128, NQ, false, false);
         if (!want_out)
@@ -321,7 +330,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
       __syncwarp();
     } else if (warp == 18) {
       // =============================== O^T products ===============================
-      if (lane == 0) {
+      if (tc::elect_one()) {
         const uint64_t dh = tc::make_desc_sw128(sbase + S::ht, 16, 1024), dp = tc::make_desc_sw128(sbase + S::pt, 16, 1024);
         if (!want_out)
           for (TileOrder o(rank, K, n_score, 0); o.own; o.next(), ++seq) {
@@ -335,18 +344,18 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           for (int ks = 0; ks < D / 16; ++ks)
             tc::mma_bf16_ss(tm_o, dh + (uint64_t)(((ks >> 2) * S::ht_blk + (ks & 3) * 32) >> 4), dp + (uint64_t)(((ks >> 2) * (NQ * 128) + (ks & 3) * 32) >> 4),
                             tc::make_idesc_bf16(128, NQ, false, false), ks > 0);
-          tc::mma_commit(BAR(R_O));
+          tc::mma_commit(BAR(R_LIN));
 #pragma unroll 1
           for (TileOrder o(rank, K, n_score, n_tiles); o.own || !o.done(); o.next(), ++seq) {
-            const uint32_t st = seq & 1;
+            const uint32_t st = seq & 1, pb = seq & (NB - 1);
             WAIT(R_VFULL + st, (seq >> 1) & 1);
-            WAIT(R_PT, seq & 1);
+            WAIT(R_PT + pb, (seq / NB) & 1);
             tc::fence_after_sync();
             const uint64_t dv = tc::make_desc_sw128(sbase + stage_v(seq), 16384, 1024);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
-              tc::mma_bf16_ss(tm_o, dv + (uint64_t)((ks * 2048) >> 4), dp + (uint64_t)((ks * 2048) >> 4), tc::make_idesc_bf16(128, NQ, true, true), 1u);
-            tc::mma_commit(BAR(R_O));
+              tc::mma_bf16_ss(tm_o, dv + (uint64_t)((ks * 2048) >> 4), dp + (uint64_t)((ks * 2048 + pb * 64) >> 4), tc::make_idesc_bf16(128, NQ, true, true), 1u);
+            tc::mma_commit(BAR(R_O + pb));
             tc::mma_commit(BAR(R_VEMPTY + st));
             if (!o.own) tc::mbar_arrive(BAR(R_VEMPTY + st));
           }
@@ -400,9 +409,10 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
 #pragma unroll
         for (int j = 0; j < HQ / 2; ++j) lpart[j] = 0;
         const uint64_t sl22 = tc::pack_f2(sl2, sl2);
+        const uint32_t nit0 = nit;
 #pragma unroll 1
         for (TileOrder o(rank, K, n_score, n_tiles); o.own || !o.done(); o.next(), ++nit) {
-          const uint32_t z = nit & 1, slot3 = nit % 3u;
+          const uint32_t z = nit & 1, slot3 = nit % 3u, pb = nit & (NB - 1);
           // what this thread's key row is: visible to every query, to none, or to the chunk's tokens from its own on
           const int blk = 2 * o.t + (t >> 6), ro = t & 63;
           int first = 1 << 20;                         // first token that sees the row
@@ -432,9 +442,11 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           if (__any_sync(0xffffffffu, mx * sl2 > kGrow) && lane == 0) X.grow[slot3][hf] = 1;
           tc::named_bar_sync(4 + hf, 128);             // the four warps of these columns
           const bool grow = *reinterpret_cast<volatile int*>(&X.grow[slot3][hf]) != 0;
-          WAIT(R_O, ev & 1);                           // the product before is complete: its weights may be overwritten, O^T moved
-          ++ev;
+          // the product that read this buffer is complete (for the first tile: the linear term, whose phi(Q) lies there)
+          if (nit == nit0) WAIT(R_LIN, chunk & 1);
+          if (nit >= NB) WAIT(R_O + pb, (nit / NB - 1) & 1);
           if (grow) {                                  // rare, uniform over the four warps
+            if (NB > 1 && nit > 0) WAIT(R_O + (pb ^ 1), ((nit - 1) / NB) & 1);   // O^T is moved: the product before, too
             tc::fence_after_sync();
 #pragma unroll
             for (int sb = 0; sb < HQ / 16; ++sb) {
@@ -483,11 +495,11 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
               lpart[(j + i) / 2] = tc::add2(lpart[(j + i) / 2], tc::pack_f2(p0, p1));
               pk[i / 2] = pack_bf16x2(p0, p1);
             }
-            *reinterpret_cast<uint4*>(sm + S::pt + tc::sw128_off(t, (hf * HQ + j) >> 3)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *reinterpret_cast<uint4*>(sm + S::pt + tc::sw128_off(t, (int)pb * 4 + ((hf * HQ + j) >> 3))) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
           tc::fence_async_smem();
           tc::fence_before_sync();
-          tc::mbar_arrive(BAR(R_PT));
+          tc::mbar_arrive(BAR(R_PT + pb));
         }
         // ---- the sums of the weights, then the outputs
 #pragma unroll
@@ -500,8 +512,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
         }
         tc::named_bar_sync(2, 256);
         if (gtid < NQ) X.inv[gtid] = 1.0f / (((X.l_s[0][gtid] + X.l_s[1][gtid]) + (X.l_s[2][gtid] + X.l_s[3][gtid])) + (X.lden[0][gtid] + X.lden[1][gtid]));
-        WAIT(R_O, ev & 1);                             // O^T is complete
-        ++ev;
+        WAIT(R_O + ((nit - 1) & (NB - 1)), ((nit - 1) / NB) & 1);   // O^T is complete
         tc::fence_after_sync();
         tc::named_bar_sync(2, 256);
 #pragma unroll
@@ -565,10 +576,10 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
             if (i < 0) i += eta;
             if ((blk - nGB) * 64 + ro < cw && i < c.r) e = cg + i;
           }
-          // (the key tile's barrier may complete again before a late warp has looked at it: the issuing thread alone must wait)
-          if (tid == 0) WAIT(R_KFULL + st, par); else tc::mbar_try_wait(BAR(R_KFULL + st), par);
+          // (the key tile's barrier may complete again before a late warp has looked at it: the issuing warp alone must wait)
+          if (warp == 0) WAIT(R_KFULL + st, par); else tc::mbar_try_wait(BAR(R_KFULL + st), par);
           tc::fence_after_sync();
-          if (tid == 0) {
+          if (warp == 0 && tc::elect_one()) {
             const uint64_t dk = tc::make_desc_sw128(sbase + stage_k(seq), 16, 1024);
 #pragma unroll
             for (int ks = 0; ks < d / 16; ++ks)
@@ -590,7 +601,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           tc::fence_before_sync();
           sync();
           tc::fence_after_sync();
-          if (tid == 0) {
+          if (warp == 0 && tc::elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks)
               tc::mma_bf16_ts(tm_p, tm_u + ks * 8, dh + (uint64_t)(((ks >> 2) * S::ht_blk + (ks & 3) * 32) >> 4), id_p, ks > 0);
@@ -709,7 +720,7 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           tc::cluster_arrive();                        // (A)
           sync();
           tc::fence_after_sync();
-          if (tid == 0) {
+          if (warp == 0 && tc::elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < d / 16; ++ks)
               tc::mma_bf16_ss(tm_u, tc::make_desc_sw128(sbase + S::fold_k + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
@@ -758,8 +769,10 @@ k_prefill_run(Layer L, Call c, int n_chunks, const __grid_constant__ RunMaps M, 
           tc::fence_before_sync();
           sync();
           tc::fence_after_sync();
-          if (tid == 0) tc::fold_product<DPL, THREE>(tm_p, sbase + S::fold_k, sbase + S::fold_v, three);
-          if (tid == 0) tc::mma_commit(BAR(R_S));
+          if (warp == 0 && tc::elect_one()) {
+            tc::fold_product<DPL, THREE>(tm_p, sbase + S::fold_k, sbase + S::fold_v, three);
+            tc::mma_commit(BAR(R_S));
+          }
           if (tid < dK * 16) load_h(tid);
           WAIT(R_S, ph_s & 1);
           ++ph_s;

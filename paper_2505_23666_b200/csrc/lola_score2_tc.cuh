@@ -37,14 +37,18 @@ struct ScoreBlocks {
 
 // TMA loads of one tile (two blocks); a block beyond the last one lies outside the ring tensor and reads as zeros.
 template <int DPL>
-__device__ __forceinline__ void score_issue_tile(uint32_t dst, const CUtensorMap* tm_g, const CUtensorMap* tm_w, int tile,
+__device__ __forceinline__ void score_issue_tile(uint32_t dst, const tc::SlotMaps* tm_g, const CUtensorMap* tm_w, int tile,
                                                  const ScoreBlocks& B, int eta, int unit, uint32_t bar) {
   constexpr int kblk = DPL / 2;
   tc::mbar_expect_tx(bar, (uint32_t)kblk * 16384u);
+  if (tile * 2 + 1 < B.nGB) {
+    tc::tma_load_slots(dst, tm_g, tile, unit, bar);
+    return;
+  }
 #pragma unroll
   for (int hb = 0; hb < 2; ++hb) {
     const int blk = tile * 2 + hb, rb = blk - B.nGB;
-    const CUtensorMap* tm = rb < 0 ? tm_g : tm_w;
+    const CUtensorMap* tm = rb < 0 ? &tm_g->block : tm_w;
     const int row = rb < 0 ? blk * 64 : (rb < B.nR1 ? B.s0 + rb * 64 : (rb < B.nR1 + B.nR2 ? (rb - B.nR1) * 64 : eta));
 #pragma unroll
     for (int cb = 0; cb < kblk; ++cb)
@@ -75,7 +79,7 @@ struct Score2Misc {
 
 template <int DPL>
 __global__ void __launch_bounds__(kSc2Threads, 1)
-k_score2_tc(Layer L, Call c, const __grid_constant__ CUtensorMap tm_gk, const __grid_constant__ CUtensorMap tm_gv,
+k_score2_tc(Layer L, Call c, const __grid_constant__ tc::SlotMaps tm_gk, const __grid_constant__ tc::SlotMaps tm_gv,
             const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv, const uint4* wt_image,
             int tiles_per_cta, int beside_attention) {
   using S = Score2Smem<DPL>;

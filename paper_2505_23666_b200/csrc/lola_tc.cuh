@@ -2,6 +2,7 @@
 // (128-byte swizzled canonical layouts), accumulators in tensor memory, mbarrier completion with
 // bounded waits.
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -36,6 +37,21 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, bool a_mn_m
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One lane of a converged warp (always the same one).  Knowing that one thread is left, the compiler hands the operands of MMAs
+// and TMA requests over without a loop over lanes: 8 MMAs take their thread 200 cycles, not 474 as with "lane == 0", a request 52
+// and not 100 (idle SM).  Taken where it measured faster: the roles of k_prefill_run and what requests tiles in k_prefill_team;
+// the issuing threads of the other kernels, whose products follow each other closely, were 1 - 4% slower with it.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t"
+      "}\n"
+      : "=r"(one));
+  return one != 0;
+}
 __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t"
@@ -226,6 +242,19 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst_smem, const void* tmap,
       "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
       ::"r"(dst_smem), "l"((uint64_t)(uintptr_t)tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
       : "memory");
+}
+// Tensor maps of a sparse cache [units][slots][d].  A tile is 128 rows of all columns, [d / 64][128 rows][128 bytes] in shared
+// memory.  A request takes its issuing thread 100 cycles on an idle SM and some 300 beside working warps, whatever its size,
+// so a tile that lies in the cache as a whole is one request, not four of 64 rows x 64 columns: eight of those a tile (keys and
+// values) held the tiles of a prefill run apart (a chunk of 8 units, d = 128: 19.6 us, with whole tiles and elect_one 18.6; 64
+// units: 28.2 and 27.7).
+struct SlotMaps {
+  CUtensorMap block;             // rank 3, boxes of 64 rows x 64 columns
+  CUtensorMap tile;              // rank 4 (column, row, block of 64 columns, unit), boxes of 128 rows x all columns
+};
+// Tile `tile` (all 128 of its rows are places of sparse-cache blocks)
+__device__ __forceinline__ void tma_load_slots(uint32_t dst_smem, const SlotMaps* m, int tile, int unit, uint32_t bar) {
+  tma_load_4d(dst_smem, &m->tile, 0, tile * 128, 0, unit, bar);
 }
 // One box of a rank-4 tensor map, shared -> global (bulk async-group completion).  Rows of the box that lie
 // outside the tensor are not written.  c0 as for the loads (16-byte aligned start); no negative coordinates.

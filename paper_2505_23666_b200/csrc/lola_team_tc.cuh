@@ -28,7 +28,10 @@ constexpr int kTeamThreads = 576;
 constexpr int kTeamMaxE = 2048;      // eligible pairs of a unit
 constexpr int kTeamMaxN = 256;       // tokens per chunk
 
-struct TeamMaps { CUtensorMap gk, gv, wk, wv, q, k, v, out; };
+struct TeamMaps {
+  tc::SlotMaps gk, gv;
+  CUtensorMap wk, wv, q, k, v, out;
+};
 
 struct TeamAttMisc {
   uint64_t bars[20];
@@ -213,7 +216,7 @@ k_prefill_team(Layer L, Call c, int n_chunks, const __grid_constant__ TeamMaps M
           tc::bulk_copy_g2s(sbase + S::stage0 + st * S::stage_bytes, wt_image + (size_t)h * kblk * 512, kblk * 8192u, BAR(TA_KFULL + st));
           ++ke;
         };
-        if (lane == 0) {
+        if (tc::elect_one()) {
           if (chunk == 0 && rank < items) start_item(rank, 0);
 #pragma unroll 1
           for (int it = rank; it < items; it += A) {
@@ -226,13 +229,16 @@ k_prefill_team(Layer L, Call c, int n_chunks, const __grid_constant__ TeamMaps M
                 if (e >= 2) WAIT((isv ? TA_VEMPTY : TA_KEMPTY) + st, ((e >> 1) & 1) ^ 1);
                 if (!ok) break;
                 tc::mbar_expect_tx(bar, (uint32_t)kblk * 16384u);
+                const uint32_t dst = sbase + S::stage0 + st * S::stage_bytes + (isv ? S::st_v : 0u);
+                const bool whole = kt * 2 + 1 < nGB;
+                if (whole) tc::tma_load_slots(dst, isv ? &M.gv : &M.gk, kt, unit, bar);
 #pragma unroll 1
-                for (int hb = 0; hb < 2; ++hb) {
+                for (int hb = whole ? 2 : 0; hb < 2; ++hb) {
                   const int blk = kt * 2 + hb;
 #pragma unroll
                   for (int cb = 0; cb < kblk; ++cb) {
-                    const uint32_t dd = sbase + S::stage0 + st * S::stage_bytes + (isv ? S::st_v : 0u) + (uint32_t)cb * 16384u + (uint32_t)hb * 8192u;
-                    if (blk < nGB) tc::tma_load_3d(dd, isv ? &M.gv : &M.gk, cb * 64, blk * 64, unit, bar);
+                    const uint32_t dd = dst + (uint32_t)cb * 16384u + (uint32_t)hb * 8192u;
+                    if (blk < nGB) tc::tma_load_3d(dd, isv ? &M.gv.block : &M.gk.block, cb * 64, blk * 64, unit, bar);
                     else if (blk < nGB + nRB) tc::tma_load_3d(dd, isv ? &M.wv : &M.wk, cb * 64, (blk - nGB) * 64, unit, bar);
                     else tc::tma_load_5d(dd, isv ? &M.v : &M.k, cb * 64, h, (blk - nGB - nRB) * 64, b, chunk, bar);   // (beyond the chunk: zeros)
                   }
@@ -245,7 +251,7 @@ k_prefill_team(Layer L, Call c, int n_chunks, const __grid_constant__ TeamMaps M
         }
         __syncwarp();
         tc::cluster_arrive();                          // (A)
-        if (lane == 0 && chunk + 1 < n_chunks && rank < items) start_item(rank, chunk + 1);
+        if (chunk + 1 < n_chunks && rank < items && tc::elect_one()) start_item(rank, chunk + 1);
         __syncwarp();
       } else if (warp == 16) {
         // =============================== MMA issuer ===============================
@@ -534,7 +540,7 @@ k_prefill_team(Layer L, Call c, int n_chunks, const __grid_constant__ TeamMaps M
       const int n_score = sel ? SB.tiles() : 0, ring0 = SB.s0;
       if (warp >= 16) {
         // =============================== tiles of group warp - 16 ===============================
-        if (lane == 0) {
+        if (tc::elect_one()) {
           const int gp = warp - 16;
 #pragma unroll 1
           for (int tile = sr + gp * N; tile < n_score; tile += 2 * N, ++en) {
