@@ -682,10 +682,10 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
   st->tensor_path = cfg->dtype == LOLA_BF16 && cfg->feat_half == 64 && !(cfg->flags & LOLA_FLAG_GENERIC_KERNELS);
   if (rc == LOLA_OK && cfg->dtype == LOLA_F32 && !(cfg->flags & LOLA_FLAG_GENERIC_KERNELS)) {
     // fp32 step as one kernel: as many blocks per unit as have an SM each, if a block's shared memory suffices
-    const int U = cfg->batch * cfg->n_kv_heads, smem_max = 227 * 1024;
+    const int U = cfg->batch * cfg->n_kv_heads, smem_max = kUnSmem;
     int K = 8;
     while (K > 1 && U * K > sms) K >>= 1;
-    if (unit_layout(L, K).total * 4 <= smem_max &&
+    if (unit_layout(L, K).total * 4 <= smem_max && cfg->sparse + cfg->max_chunk <= 32 * kUnGroup &&
         (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_run<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)
                               : cudaFuncSetAttribute(k_unit_run<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) == cudaSuccess)
       st->unit_blocks = K;

@@ -6,14 +6,18 @@
 // chain of four kernels with a block per 16 or 32 rows it took 167 us, nearly all of it launches, round trips to
 // memory between dependent phases and a quadratic selection.  Here a unit's H, s, W and positions stay in shared
 // memory for the whole run and the phases of a chunk are separated by cluster barriers:
-//   A  every block: its share of E = sparse cache + leaving pairs: feature map (kept), Eq. 10 score, sent to all
-//      blocks of the cluster; then (prefill) its share of the queries: Eq. 14 against the H, s of the chunk's start
+//   A  every block, two groups of 256 threads side by side:
+//        its share of E = sparse cache + leaving pairs: feature map (kept), Eq. 10 score, sent to all blocks of the cluster
+//        (prefill) its share of the queries: Eq. 14 against the H, s of the chunk's start
 //   -- barrier: all scores are everywhere, nobody reads the old H or ring any more
 //   B  every block for itself: the selection (Eq. 12); the feature rows of the folded pairs come from the blocks that
 //      computed them, each block folds its D / K rows of H and s (Eq. 13) and sends them to the others
 //   -- barrier: the folded pairs have been read, their slots may be overwritten
 //   C  moves into the sparse cache and window roll, a warp per token
 //   -- barrier; (generation step) Eq. 14 on the updated memories
+// One group after the other a chunk took 27.0 us, side by side 22.2 (4 units of 192 pairs, 64 tokens, d = 64; 64 units of 300 pairs 93.7
+// and 74.4): the two share the SM's path to shared memory, which the products keep busy.  Where the scratch does not fit twice the
+// attention waits for the scores.
 // K is the largest of 8, 4, 2, 1 that lets every block have an SM of its own: more blocks only shorten the phases.
 // The body of the chunk loop has to stay in the instruction cache: with everything unrolled (226 KB of code) a chunk
 // took 33 us, three quarters of it instruction fetch.  Hence short rolled loops, no integer division inside them and
@@ -28,10 +32,12 @@
 
 namespace lola {
 
-constexpr int kUnThreads = 256;
+constexpr int kUnThreads = 512;   // two groups of 256: scoring and attention side by side, then both
+constexpr int kUnGroup = 256;
+constexpr int kUnSmem = 227 * 1024;
 constexpr int kUnRows = 32;    // members of E per scoring tile: thread = 2 rows x 4 columns of a 32 x 64 product
 constexpr int kUnQ = 8;        // query rows per batch (one per warp in the softmax)
-constexpr int kUnKeys = 256;   // keys per tile (one per thread in q.k)
+constexpr int kUnKeys = 256;   // keys per tile
 constexpr int kUnFold = 64;    // folded pairs per pass
 constexpr int kUnSrcFloats = 40;
 
@@ -39,11 +45,13 @@ struct UnitLayout {            // shared memory of k_unit_run, offsets in floats
   int fp, dp;                  // F and D rounded up to a multiple of 4 (zero padding)
   int jn, jsh;                 // rows of H a block folds, and the power of two that covers them
   int phi_ld;
-  int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, dst, sel, src, total;
+  int serial;                  // the two groups share one scratch, scoring first (it does not fit twice)
+  int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, dst, sel, src, part, total;
 };
 
-LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
+LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
   UnitLayout Y{};
+  Y.serial = serial;
   const int d = L.d, nE = L.lam + L.cmax, rp = (nE + K - 1) / K;
   Y.fp = (L.F + 3) & ~3;
   Y.dp = (L.D + 3) & ~3;
@@ -56,23 +64,24 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
   Y.H = take(Y.dp * d);
   Y.s = take(Y.dp);
   Y.phi = take((rp + kUnRows - 1) / kUnRows * kUnRows * Y.phi_ld);
-  // the three phases of a chunk take turns in the same space
+  // the phases of a chunk take turns in the same space
   const int phase0 = o;
   Y.xs = take(kUnRows * (d + 4));
   Y.den = take(kUnRows);
   int end = o;
-  o = phase0;
+  if (serial) o = phase0;
   Y.q = take(kUnQ * d);
   Y.pq = take(Y.dp * kUnQ);
   Y.z = take(kUnQ * kUnKeys);              // (first the queries' u, 128 floats a row)
   Y.p = take(kUnKeys * kUnQ);
   Y.vptr = take(kUnKeys * 2);
-  Y.red = take(kUnThreads / 32 * kUnQ * 64);
+  Y.red = take(kUnGroup / 32 * kUnQ * 64);
   Y.row = take(kUnQ * 3);
   end = end > o ? end : o;
   o = phase0;
   Y.vf = take(kUnFold * d);
   Y.pf = take(kUnFold * Y.jn);
+  Y.part = take(kUnGroup * 4);
   o = end > o ? end : o;
   Y.key = take(nE);
   Y.pos = take(nE);
@@ -84,6 +93,11 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
   Y.src = take(kUnSrcFloats);
   Y.total = o;
   return Y;
+}
+
+LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
+  const UnitLayout Y = unit_layout(L, K, 0);
+  return Y.total * 4 <= kUnSmem ? Y : unit_layout(L, K, 1);
 }
 
 // Where the rows of a unit lie during one chunk (shared memory; every pointer is the unit's own first row).
@@ -115,37 +129,43 @@ __device__ __forceinline__ void unit_key(const UnitSrc& U, int i, int d, const f
   } else { kp = U.k + (size_t)(i - U.att_wn) * U.kstep; vp = U.v + (size_t)(i - U.att_wn) * U.kstep; }
 }
 
-// The feature map of two rows by one warp, side by side (a row alone is a chain of reductions, exponentials and
-// divisions): u[r * u_ld + f] -> out[r * o_row + j * o_col], j over the D features; returns phi . ss of the two rows.
-__device__ __noinline__ float2 unit_phi2(const float* u, int u_ld, float* out, int o_row, int o_col, int F, int kind, const float* ss) {
+// The feature map of R rows by one warp, side by side (a row alone is a chain of reductions, exponentials and
+// divisions), N features of each sign per lane (F <= 32 N): u[r * u_ld + f] -> out[r * o_row + j * o_col], j over the D features;
+// ds[r] = phi . ss.
+template <int R, int N>
+__device__ __noinline__ void unit_phi(const float* u, int u_ld, float* out, int o_row, int o_col, int F, int kind, const float* ss, float* ds_out) {
   const int lane = threadIdx.x & 31;
-  float mx[2] = {-CUDART_INF_F, -CUDART_INF_F}, mn[2] = {CUDART_INF_F, CUDART_INF_F}, s1[2] = {1.f, 1.f}, s2[2] = {1.f, 1.f}, ds[2] = {0.f, 0.f};
-  float a[2][4];
+  float mx[R], mn[R], s1[R], s2[R], ds[R];
+  float a[R][N];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int r = 0; r < R; ++r) { mx[r] = -CUDART_INF_F; mn[r] = CUDART_INF_F; s1[r] = s2[r] = 1.f; ds[r] = 0.f; }
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
       const bool in = lane + 32 * i < F;
       a[r][i] = in ? u[r * u_ld + lane + 32 * i] : 0.f;
       if (in) { mx[r] = fmaxf(mx[r], a[r][i]); mn[r] = fminf(mn[r], a[r][i]); }
     }
   __syncwarp();                                        // (out may lie over u)
-  if (kind == 1) { mx[0] = mx[1] = mn[0] = mn[1] = 0.f; }
-  else {
+  if (kind == 1) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) mx[r] = mn[r] = 0.f;
+  } else {
 #pragma unroll 1
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
+      for (int r = 0; r < R; ++r) {
         mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], o));
         mn[r] = fminf(mn[r], __shfl_xor_sync(0xffffffffu, mn[r], o));
       }
   }
-  float p[2][4], q[2][4];
+  float p[R][N], q[R][N];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < R; ++r) {
     float t1 = 0.f, t2 = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < N; ++i) {
       p[r][i] = q[r][i] = 0.f;
       if (lane + 32 * i < F) { p[r][i] = expf(a[r][i] - mx[r]); q[r][i] = expf(mn[r] - a[r][i]); }
       t1 += p[r][i];
@@ -157,15 +177,15 @@ __device__ __noinline__ float2 unit_phi2(const float* u, int u_ld, float* out, i
 #pragma unroll 1
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
+      for (int r = 0; r < R; ++r) {
         s1[r] += __shfl_xor_sync(0xffffffffu, s1[r], o);
         s2[r] += __shfl_xor_sync(0xffffffffu, s2[r], o);
       }
   }
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < N; ++i) {
       const int f = lane + 32 * i;
       if (f < F) {
         const float x = p[r][i] / s1[r], y = q[r][i] / s2[r];
@@ -177,8 +197,10 @@ __device__ __noinline__ float2 unit_phi2(const float* u, int u_ld, float* out, i
 #pragma unroll 1
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int r = 0; r < 2; ++r) ds[r] += __shfl_xor_sync(0xffffffffu, ds[r], o);
-  return make_float2(ds[0], ds[1]);
+    for (int r = 0; r < R; ++r) ds[r] += __shfl_xor_sync(0xffffffffu, ds[r], o);
+  if (lane == 0)
+#pragma unroll
+    for (int r = 0; r < R; ++r) ds_out[r] = ds[r];
 }
 
 // Eq. 14 for the query rows of one block of the cluster, in batches of kUnQ rows.  Key tile: a thread's whole key row
@@ -186,8 +208,9 @@ __device__ __noinline__ float2 unit_phi2(const float* u, int u_ld, float* out, i
 // linear term is the accumulator's first summand, with the weight of a key whose score is 0.
 template <int DPL>
 __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const UnitLayout& Y, float* sm, UnitSrc& U, int b, int h, int rank, int K) {
-  constexpr int d = DPL * 32, NC = d / 64, KG = kUnThreads / 16;     // NC: 64-column blocks, KG: key groups
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int d = DPL * 32, NC = d / 64, KG = kUnGroup / 16;     // NC: 64-column blocks, KG: key groups
+  const int tid = threadIdx.x & (kUnGroup - 1), warp = tid >> 5, lane = tid & 31;
+  auto sync = [] { tc::named_bar_sync(2, kUnGroup); };
   const int nrows = L.g * c.nq, NK = c.att_g + c.att_wn + c.att_chunk, chunk0 = c.att_g + c.att_wn;
   const float* Hs = sm + Y.H;
   float *qs = sm + Y.q, *pq = sm + Y.pq, *zs = sm + Y.z, *ps = sm + Y.p, *red = sm + Y.red, *rw = sm + Y.row;
@@ -200,33 +223,38 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
       U.tok_of[tid] = tok;
       U.out_row[tid] = row < nrows ? (b * c.nq + tok) * L.Hq + h * L.g + hl : -1;
     }
-    __syncthreads();
+    sync();
     if (tid < kUnQ * (d / 4)) {
       const int rr = tid / (d / 4), row = U.out_row[rr];
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       if (row >= 0) x = *reinterpret_cast<const float4*>((const float*)c.q + (size_t)row * d + tid % (d / 4) * 4);
       *reinterpret_cast<float4*>(qs + tid * 4) = x;
     }
-    __syncthreads();
+    sync();
     // u = q W: warp = row, 4 features per lane and pass; then the feature map of two rows per warp, transposed into pq
+    const bool two = Y.fp <= 64;                       // (half a warp has all features: the other half takes half of the inner dimension)
 #pragma unroll 1
-    for (int f = lane * 4; f < Y.fp; f += 128) {
-      const float *x = qs + warp * d, *w = sm + Y.W + f;
+    for (int f = (two ? lane & 15 : lane) * 4; f < Y.fp; f += 128) {
+      const int jb = two && lane >= 16 ? d / 2 : 0, jn = two ? d / 2 : d;
+      const float *x = qs + warp * d + jb, *w = sm + Y.W + jb * Y.fp + f;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
-      for (int j = 0; j < d; ++j) {
+      for (int j = 0; j < jn; ++j) {
         const float4 wv = *reinterpret_cast<const float4*>(w + j * Y.fp);
         const float xj = x[j];
         a.x = fmaf(xj, wv.x, a.x); a.y = fmaf(xj, wv.y, a.y); a.z = fmaf(xj, wv.z, a.z); a.w = fmaf(xj, wv.w, a.w);
       }
-      *reinterpret_cast<float4*>(zs + warp * 128 + f) = a;
+      if (two) {
+        const unsigned m16 = (1u << min(16, Y.fp / 4)) - 1u, both = m16 | m16 << 16;
+        a.x += __shfl_xor_sync(both, a.x, 16); a.y += __shfl_xor_sync(both, a.y, 16);
+        a.z += __shfl_xor_sync(both, a.z, 16); a.w += __shfl_xor_sync(both, a.w, 16);
+      }
+      if (!two || lane < 16) *reinterpret_cast<float4*>(zs + warp * 128 + f) = a;
     }
-    __syncthreads();
-    if (warp < kUnQ / 2) {
-      const float2 ds = unit_phi2(zs + warp * 256, 128, pq + warp * 2, 1, kUnQ, L.F, L.phi_kind, sm + Y.s);
-      if (lane == 0) { rw[2 * kUnQ + warp * 2] = ds.x; rw[2 * kUnQ + warp * 2 + 1] = ds.y; }
-    }
-    __syncthreads();
+    sync();
+    if (two) unit_phi<1, 2>(zs + warp * 128, 128, pq + warp, 1, kUnQ, L.F, L.phi_kind, sm + Y.s, rw + 2 * kUnQ + warp);
+    else unit_phi<1, 4>(zs + warp * 128, 128, pq + warp, 1, kUnQ, L.F, L.phi_kind, sm + Y.s, rw + 2 * kUnQ + warp);
+    sync();
     float m = 0.f, l = (c.att_flags & 1) ? 0.f : rw[2 * kUnQ + warp];   // this warp's row: stabiliser max(0, max z), sum of the weights
     float acc[NC][kUnQ][4];
 #pragma unroll
@@ -252,36 +280,60 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
     }
 #pragma unroll 1
     for (int kt = 0; kt < NK; kt += kUnKeys) {
-      const int idx = kt + tid, nk = min(kUnKeys, NK - kt);
-      float z[kUnQ];
-#pragma unroll
-      for (int r = 0; r < kUnQ; ++r) z[r] = 0.f;
-      if (idx < NK) {
-        const float *kp, *vp;
-        unit_key(U, idx, d, kp, vp);
-        vptr[tid] = vp;
+      const int nk = min(kUnKeys, NK - kt);
+      // q.k: four lanes per key, four keys per thread (two at a time where a thread holds 128 columns).  A lane takes every fourth 16 bytes of a key (a whole row per thread touches a
+      // line per lane and load); the queries' pieces serve all its keys; the lanes' sums meet in a reduce-scatter, two queries a lane
+      constexpr int NP = DPL == 4 ? 2 : 4;
+      const int sub = tid & 3;
 #pragma unroll 1
-        for (int j0 = 0; j0 < d; j0 += 32) {
-          float4 kv[8];
+      for (int k0 = tid >> 2; k0 < kUnKeys; k0 += NP * (kUnGroup / 4)) {
+        float z[NP][kUnQ];
+        const float* kp[NP];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) kv[j] = *reinterpret_cast<const float4*>(kp + j0 + j * 4);
+        for (int p = 0; p < NP; ++p) {
+          const int kb = k0 + p * (kUnGroup / 4);
+          const float *kk = qs, *vp = qs;              // (beyond the last key: masked)
+          if (kb < nk) unit_key(U, kt + kb, d, kk, vp);
+          kp[p] = kk + sub * 4;
+          if (sub == 0) vptr[kb] = vp;
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
+          for (int r = 0; r < kUnQ; ++r) z[p][r] = 0.f;
+        }
+#pragma unroll 1
+        for (int j0 = 0; j0 < d; j0 += 64) {
+          float4 kv[NP][4];
+#pragma unroll
+          for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) kv[p][j] = *reinterpret_cast<const float4*>(kp[p] + j0 + j * 16);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int r = 0; r < kUnQ; ++r) {
-              const float4 qv = *reinterpret_cast<const float4*>(qs + r * d + j0 + j * 4);
-              z[r] = fmaf(qv.x, kv[j].x, z[r]);
-              z[r] = fmaf(qv.y, kv[j].y, z[r]);
-              z[r] = fmaf(qv.z, kv[j].z, z[r]);
-              z[r] = fmaf(qv.w, kv[j].w, z[r]);
+              const float4 qv = *reinterpret_cast<const float4*>(qs + r * d + j0 + j * 16 + sub * 4);
+#pragma unroll
+              for (int p = 0; p < NP; ++p)
+                z[p][r] = fmaf(qv.w, kv[p][j].w, fmaf(qv.z, kv[p][j].z, fmaf(qv.y, kv[p][j].y, fmaf(qv.x, kv[p][j].x, z[p][r]))));
             }
         }
-      }
-      const int ci = idx - chunk0;
 #pragma unroll
-      for (int r = 0; r < kUnQ; ++r)
-        zs[r * kUnKeys + tid] = idx < NK && (ci < 0 || ci <= U.tok_of[r]) ? z[r] * L.scale : -CUDART_INF_F;
-      __syncthreads();
+        for (int p = 0; p < NP; ++p) {
+          const int kb = k0 + p * (kUnGroup / 4), ci = kt + kb - chunk0;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const float keep = sub & 2 ? z[p][r + 4] : z[p][r], give = sub & 2 ? z[p][r] : z[p][r + 4];
+            z[p][r] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+          }
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const float keep = sub & 1 ? z[p][r + 2] : z[p][r], give = sub & 1 ? z[p][r] : z[p][r + 2];
+            const float zz = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+            const int row = (sub & 2) * 2 + (sub & 1) * 2 + r;
+            zs[row * kUnKeys + kb] = kb < nk && (ci < 0 || ci <= U.tok_of[row]) ? zz * L.scale : -CUDART_INF_F;
+          }
+        }
+      }
+      sync();
       float4 vv[8];                                    // the first half of the first column block's values, ahead of the softmax
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -305,7 +357,7 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
         m = mt;
         if (lane == 0) rw[warp] = alpha;
       }
-      __syncthreads();
+      sync();
 #pragma unroll
       for (int r = 0; r < kUnQ; ++r) {
         const float alpha = rw[r];
@@ -326,7 +378,7 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
 #pragma unroll
           for (int i = 0; i < 8; ++i) add(nc, vv[i], ps + (k0 + i * KG) * kUnQ);
         }
-      __syncthreads();
+      sync();
     }
     if (lane == 0) rw[kUnQ + warp] = l;
     // the 16 key groups meet: two inside a warp, then eight warps through shared memory
@@ -339,22 +391,22 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
         if (lane < 16)
           *reinterpret_cast<float4*>(red + (warp * kUnQ + r) * 64 + c4) = make_float4(acc[nc][r][0], acc[nc][r][1], acc[nc][r][2], acc[nc][r][3]);
       }
-      __syncthreads();
+      sync();
 #pragma unroll 1
-      for (int i = tid; i < kUnQ * 64; i += kUnThreads) {
+      for (int i = tid; i < kUnQ * 64; i += kUnGroup) {
         const int r = i >> 6, cc = i & 63;
         float a = 0.f;
 #pragma unroll
-        for (int w = 0; w < kUnThreads / 32; ++w) a += red[(w * kUnQ + r) * 64 + cc];
+        for (int w = 0; w < kUnGroup / 32; ++w) a += red[(w * kUnQ + r) * 64 + cc];
         if (U.out_row[r] >= 0) ((float*)c.out)[(size_t)U.out_row[r] * d + nc * 64 + cc] = a / rw[kUnQ + r];
       }
-      __syncthreads();
+      sync();
     }
   }
 }
 
 template <int DPL>
-__global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_chunks, int decode, UnitLayout Y) {
+__global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int n_chunks, int decode, UnitLayout Y) {
   namespace co = cooperative_groups;
   constexpr int d = DPL * 32, d4 = d / 4;
   extern __shared__ __align__(16) float sm[];
@@ -362,7 +414,8 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
   const int K = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int unit = blockIdx.x / K, b = unit / L.Hkv, h = unit % L.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tx = tid & 15, ty = tid >> 4;
+  const int grp = tid >> 8, gt = tid & (kUnGroup - 1), tx = gt & 15, ty = gt >> 4;
+  auto gsync = [] { tc::named_bar_sync(1, kUnGroup); };   // the scoring group
   float *Ws = sm + Y.W, *Hs = sm + Y.H, *ss = sm + Y.s, *phi = sm + Y.phi, *xs = sm + Y.xs, *den = sm + Y.den, *vf = sm + Y.vf, *pf = sm + Y.pf;
   unsigned* key = reinterpret_cast<unsigned*>(sm + Y.key);
   int *pos = reinterpret_cast<int*>(sm + Y.pos), *cand = reinterpret_cast<int*>(sm + Y.cand), *fold = reinterpret_cast<int*>(sm + Y.fold),
@@ -421,9 +474,9 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
     __syncthreads();
     // ---- A: feature rows and scores of this block's members of E
 #pragma unroll 1
-    for (int t0 = 0; t0 < ne; t0 += kUnRows) {
+    for (int t0 = 0; t0 < (grp == 0 ? ne : 0); t0 += kUnRows) {
 #pragma unroll 2
-      for (int i = tid; i < kUnRows * d4; i += kUnThreads) {
+      for (int i = gt; i < kUnRows * d4; i += kUnGroup) {
         const int row = i / d4, c4 = i % d4;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (t0 + row < ne) {
@@ -433,11 +486,11 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
         }
         *reinterpret_cast<float4*>(xs + row * (d + 4) + c4 * 4) = x;
       }
-      __syncthreads();
+      gsync();
       float* prow = phi + (size_t)(t0 + 2 * ty) * Y.phi_ld;         // this thread's two feature rows
       // a 2 x 4 tile of x m per thread: x rows in shared memory (ldx floats apart), m [k][ldm]
       auto tile = [&](const float* x, int ldx, const float* m, int ldm, int kk, float (&a)[2][4]) {
-#pragma unroll 2
+#pragma unroll 4
         for (int k = 0; k < kk; k += 4) {
           const float4 x0 = *reinterpret_cast<const float4*>(x + k), x1 = *reinterpret_cast<const float4*>(x + ldx + k);
           const float xa[4] = {x0.x, x0.y, x0.z, x0.w}, xb[4] = {x1.x, x1.y, x1.z, x1.w};
@@ -465,15 +518,16 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
 #pragma unroll
           for (int q = 0; q < d / 64; ++q) val[rr][q] = *reinterpret_cast<const float4*>(vp + q * 64 + tx * 4);
         }
-      __syncthreads();
-#pragma unroll 1
-      for (int row = warp * 2; row < kUnRows; row += kUnThreads / 16) {
-        float* f = phi + (size_t)(t0 + row) * Y.phi_ld;
-        const float2 ds = unit_phi2(f, Y.phi_ld, f, Y.phi_ld, 1, L.F, L.phi_kind, ss);
-        if (lane == 0) { den[row] = ds.x; den[row + 1] = ds.y; }
-        if (lane < Y.dp - L.D) f[L.D + lane] = f[Y.phi_ld + L.D + lane] = 0.f;
+      gsync();
+      {
+        float* f = phi + (size_t)(t0 + warp * 4) * Y.phi_ld;
+        if (L.F <= 64) unit_phi<4, 2>(f, Y.phi_ld, f, Y.phi_ld, 1, L.F, L.phi_kind, ss, den + warp * 4);
+        else unit_phi<4, 4>(f, Y.phi_ld, f, Y.phi_ld, 1, L.F, L.phi_kind, ss, den + warp * 4);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (lane < Y.dp - L.D) f[r * Y.phi_ld + L.D + lane] = 0.f;
       }
-      __syncthreads();
+      gsync();
       if (scored) {
         float err[2] = {0.f, 0.f};
 #pragma unroll
@@ -503,9 +557,10 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
           }
         }
       }
-      __syncthreads();
+      gsync();
     }
-    if (c.out && (!decode || it == 1)) unit_attend<DPL>(L, c, Y, sm, U, b, h, rank, K);
+    if (Y.serial && ne > 0 && c.out && (!decode || it == 1)) __syncthreads();
+    if (grp == 1 && c.out && (!decode || it == 1)) unit_attend<DPL>(L, c, Y, sm, U, b, h, rank, K);
     if (decode && it == 1) break;
     cl.sync();
     // ---- B: which pairs fold, which leaving pairs stay
@@ -566,8 +621,9 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
     } else if (scored) {
       for (int i = tid; i < c.r; i += kUnThreads) pos[cg + i] = c.r_pos0 + i;
       __syncthreads();
-      select_lists<kUnThreads>(key, [&](int e) { return pos[e]; }, cand, mark, nE, nF, cg,
-                               fold, S, tid, [] { __syncthreads(); }, [&](int i, int to) { dst[i] = to; }, [] {});
+      if (grp == 0)
+        select_lists<kUnGroup>(key, [&](int e) { return pos[e]; }, cand, mark, nE, nF, cg,
+                               fold, S, tid, gsync, [&](int i, int to) { dst[i] = to; }, [] {});
       __syncthreads();
       if (rank == 0 && tid == 0) {
         L.thr[(size_t)unit * 2 + 0] = __uint_as_float(S.min_keep);
@@ -612,19 +668,33 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
           if (row + q * rstep < nb && jj < jn) pf[(row + q * rstep) * Y.jn + jj] = x[q];
       }
       __syncthreads();
+      // (where one group has all entries, the groups take half of the pairs each)
+      const bool halves = jn * d4 <= kUnGroup;
+      const int fb = halves && grp == 1 ? nb / 2 : 0, fe = halves && grp == 0 ? nb / 2 : nb;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-      for (int i = tid; i < jn * d4; i += kUnThreads) {
+      for (int i = halves ? gt : tid; i < jn * d4; i += kUnThreads) {
         const int j = i / d4, c4 = i % d4;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-        for (int f = 0; f < nb; ++f) {
+        for (int f = fb; f < fe; ++f) {
           const float p = pf[f * Y.jn + j];
           const float4 v = *reinterpret_cast<const float4*>(vf + f * d + c4 * 4);
           a.x = fmaf(p, v.x, a.x); a.y = fmaf(p, v.y, a.y); a.z = fmaf(p, v.z, a.z); a.w = fmaf(p, v.w, a.w);
         }
+        if (halves) break;
         float4* hp = reinterpret_cast<float4*>(Hs + (size_t)(j0 + j) * d + c4 * 4);
         float4 hv = *hp;
         hv.x += a.x; hv.y += a.y; hv.z += a.z; hv.w += a.w;
+        *hp = hv;
+      }
+      if (halves && grp == 1) *reinterpret_cast<float4*>(sm + Y.part + gt * 4) = a;
+      if (halves) __syncthreads();
+      if (halves && grp == 0 && gt < jn * d4) {
+        const float4 o = *reinterpret_cast<const float4*>(sm + Y.part + gt * 4);
+        float4* hp = reinterpret_cast<float4*>(Hs + (size_t)j0 * d + gt * 4);
+        float4 hv = *hp;
+        hv.x += a.x + o.x; hv.y += a.y + o.y; hv.z += a.z + o.z; hv.w += a.w + o.w;
         *hp = hv;
       }
       if (tid < jn) {
@@ -638,12 +708,12 @@ __global__ void __launch_bounds__(kUnThreads) k_unit_run(Layer L, Call c, int n_
     if (nF > 0 && !one) {
       folded = true;
 #pragma unroll 1
-      for (int r = 1; r < K; ++r) {                                   // the folded rows of H, s to the other blocks
+      for (int r = 1 + grp; r < K; r += 2) {                          // the folded rows of H, s to the other blocks
         const int to = (rank + r) & (K - 1);
         float* Hr = cl.map_shared_rank(Hs, to);
-        for (int i = tid; i < jn * d4; i += kUnThreads)
+        for (int i = gt; i < jn * d4; i += kUnGroup)
           *reinterpret_cast<float4*>(Hr + (size_t)j0 * d + i * 4) = *reinterpret_cast<const float4*>(Hs + (size_t)j0 * d + i * 4);
-        if (tid < jn) cl.map_shared_rank(ss, to)[j0 + tid] = ss[j0 + tid];
+        if (gt < jn) cl.map_shared_rank(ss, to)[j0 + gt] = ss[j0 + gt];
       }
       cl.sync();
     }
