@@ -102,8 +102,10 @@ __device__ __forceinline__ void select_body(const Layer& L, const Call& c, uint8
     X.pos[e] = e < cg ? L.gpos[(size_t)unit * lam + e] : c.r_pos0 + (e - cg);
   }
   __syncthreads();
-  select_lists<kUp2Threads>(X.key, [&](int e) { return X.pos[e]; }, X.cand, X.mark, nE, nF, cg,
-                            X.fold_e, X.scratch, tid, [] { __syncthreads(); }, [&](int i, int to) { L.move_dst[lo + i] = to; }, [] {});
+  if (tid < 256)                                       // (faster than with all threads; see select_lists)
+    select_lists<256>(X.key, [&](int e) { return X.pos[e]; }, X.cand, X.mark, nE, nF, cg,
+                      X.fold_e, X.scratch, tid, [] { tc::named_bar_sync(5, 256); }, [&](int i, int to) { L.move_dst[lo + i] = to; }, [] {});
+  __syncthreads();
   // the lists leave through the state's work-list arrays
   for (int i = tid; i < nF; i += kUp2Threads) L.fold_idx[lo + i] = X.fold_e[i];
   if (tid == 0) {
