@@ -85,12 +85,19 @@ StateLayout make_layout(const lola_config& c) {
 inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
 // The state as it is before the first token: zeros, and all ones in three byte ranges of it.  One pass: as four fills by the driver a
-// reset took 10 - 14 us (states of 1 - 17 MB), as one kernel 4 - 8.
+// reset took 10 - 14 us (states of 1 - 17 MB; 52 at 273 MB), as one kernel 4 - 6 (46).
 struct ResetRanges { size_t a0, a1, b0, b1, c0, c1; };
 __global__ void __launch_bounds__(512) k_reset(uint4* base, size_t units, ResetRanges R) {
-  for (size_t i = (size_t)blockIdx.x * 512 + threadIdx.x; i < units; i += (size_t)gridDim.x * 512) {
-    auto word = [&](size_t x) { return (x >= R.a0 && x < R.a1) || (x >= R.b0 && x < R.b1) || (x >= R.c0 && x < R.c1) ? 0xffffffffu : 0u; };
-    base[i] = make_uint4(word(i * 16), word(i * 16 + 4), word(i * 16 + 8), word(i * 16 + 12));
+  auto word = [&](size_t x) { return (x >= R.a0 && x < R.a1) || (x >= R.b0 && x < R.b1) || (x >= R.c0 && x < R.c1) ? 0xffffffffu : 0u; };
+  for (size_t t0 = (size_t)blockIdx.x * 1024; t0 < units; t0 += (size_t)gridDim.x * 1024) {   // 16 KB at a time
+    const size_t lo = t0 * 16, hi = lo + 16384;
+    const bool plain = (hi <= R.a0 || lo >= R.a1) && (hi <= R.b0 || lo >= R.b1) && (hi <= R.c0 || lo >= R.c1);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const size_t i = t0 + x * 512 + threadIdx.x;
+      if (i >= units) break;
+      base[i] = plain ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(word(i * 16), word(i * 16 + 4), word(i * 16 + 8), word(i * 16 + 12));
+    }
   }
 }
 
@@ -752,7 +759,7 @@ int lola_reset_state(lola_state* st, void* stream) {
   const StateLayout& y = st->lay;
   const ResetRanges R{y.gpos, y.gpos + U * c.sparse * 4, y.score, y.score + U * (c.sparse + c.max_chunk) * 4, y.thr, y.thr + U * 2 * 4};
   const size_t units = y.wt / 16;
-  k_reset<<<(unsigned)std::min<size_t>((units + 511) / 512, (size_t)st->sms * 4), 512, 0, s>>>((uint4*)st->base, units, R);
+  k_reset<<<(unsigned)std::min<size_t>((units + 1023) / 1024, (size_t)st->sms * 4), 512, 0, s>>>((uint4*)st->base, units, R);
   if (cudaGetLastError() != cudaSuccess) return LOLA_ERR_CUDA;
   st->n_seen = 0;
   return LOLA_OK;
