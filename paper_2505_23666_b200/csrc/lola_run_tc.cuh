@@ -5,7 +5,7 @@
 // latency (a unit's chunk is 0.17 GFLOP).  As three dependent launches it took 24 us (d = 64) to 34 us (d = 128) a
 // chunk with most SMs idle at small batches: every launch sets up its operands again (H, W, tensor memory, 4 - 5 us),
 // runs through 50 - 65 KB of cold code and hands lists over through memory.  Here the set-up happens once per run and
-// the code stays in the instruction cache: 15 us (d = 64) and 21 us (d = 128) a chunk of 8 units.  Each block has two
+// the code stays in the instruction cache: 13 us (d = 64) and 18.6 us (d = 128) a chunk of 8 units.  Each block has two
 // groups of 256 threads that work side by side:
 //
 //   score group (warps 0-7)       the tiles of E this block owns: U = K W, feature map, [P | den] = phi [H | s_hi s_lo],

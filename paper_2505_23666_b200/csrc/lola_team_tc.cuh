@@ -8,8 +8,8 @@
 //
 // What bounds it: as three dependent launches a chunk of 64 tokens of 64 units took 34.5 us (d = 128, 896 pairs): attention
 // 24 us beside scoring and selection 25 us, then the fold 8.5 us, each with its own set-up.  Here the set-up happens
-// once, the fold runs beside the attention, and only the moves of pairs wait for it: 29 us a chunk in a run (chunks of 256
-// tokens, 16 units: 51 -> 31 us).  Per chunk the cluster meets at an
+// once, the fold runs beside the attention, and only the moves of pairs wait for it: 27 us a chunk in a run (chunks of 256
+// tokens, 16 units: 51 -> 30 us).  Per chunk the cluster meets at an
 // mbarrier that counts the scores (scoring blocks), at a cluster barrier (A) when every block has read all it needs of
 // the old memories, and at one when the new memories are written.
 // Every wait on an mbarrier is bounded; a wait that runs out sets bit 512 of the status word.

@@ -15,8 +15,8 @@
 //   -- barrier: the folded pairs have been read, their slots may be overwritten
 //   C  moves into the sparse cache and window roll, a warp per token
 //   -- barrier; (generation step) Eq. 14 on the updated memories
-// One group after the other a chunk took 27.0 us, side by side 22.2 (4 units of 192 pairs, 64 tokens, d = 64; 64 units of 300 pairs 93.7
-// and 74.4): the two share the SM's path to shared memory, which the products keep busy.  Where the scratch does not fit twice the
+// One group after the other a chunk took 27.0 us, side by side 22.2 (4 units of 192 pairs, 64 tokens, d = 64; 16 units of 364 pairs, two
+// heads, 93.7 and 74.4): the two share the SM's path to shared memory, which the products keep busy.  Where the scratch does not fit twice the
 // attention waits for the scores.
 // K is the largest of 8, 4, 2, 1 that lets every block have an SM of its own: more blocks only shorten the phases.
 // The body of the chunk loop has to stay in the instruction cache: with everything unrolled (226 KB of code) a chunk
