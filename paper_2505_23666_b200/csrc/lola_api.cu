@@ -702,7 +702,7 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
     const int U = cfg->batch * cfg->n_kv_heads, smem_max = kUnSmem;
     int K = 8;
     while (K > 1 && U * K > sms) K >>= 1;
-    if (unit_layout(L, K).total * 4 <= smem_max && cfg->sparse + cfg->max_chunk <= 32 * kUnGroup &&
+    if (unit_layout(L, K).total * 4 <= smem_max &&
         (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_run<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)
                               : cudaFuncSetAttribute(k_unit_run<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) == cudaSuccess)
       st->unit_blocks = K;

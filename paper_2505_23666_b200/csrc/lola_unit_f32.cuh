@@ -49,6 +49,9 @@ struct UnitLayout {            // shared memory of k_unit_run, offsets in floats
   int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, dst, sel, src, part, total;
 };
 
+// Does one group of threads have all entries of a block's rows of H?  The groups then take half of the folded pairs each.
+LOLA_HD inline bool unit_fold_halves(int jn, int d) { return jn * (d / 4) <= kUnGroup; }
+
 LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
   UnitLayout Y{};
   Y.serial = serial;
@@ -81,15 +84,18 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
   o = phase0;
   Y.vf = take(kUnFold * d);
   Y.pf = take(kUnFold * Y.jn);
-  Y.part = take(kUnGroup * 4);
+  if (unit_fold_halves(Y.jn, d)) Y.part = take(kUnGroup * 4);
+  end = end > o ? end : o;
+  // the selection is over when the folded pairs come in; only its first value row is there beside it (the fold of one pair)
+  o = Y.vf + d;
+  Y.sel = take((int)(sizeof(SelectScratch) + 3) / 4);
+  Y.cand = take(nE);
+  Y.mark = take((nE + 3) / 4);
   o = end > o ? end : o;
   Y.key = take(nE);
   Y.pos = take(nE);
-  Y.cand = take(nE);
-  Y.mark = take((nE + 3) / 4);
   Y.fold = take(L.cmax);
   Y.dst = take(L.cmax);
-  Y.sel = take((int)(sizeof(SelectScratch) + 3) / 4);
   Y.src = take(kUnSrcFloats);
   Y.total = o;
   return Y;
@@ -621,14 +627,15 @@ __global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int
     } else if (scored) {
       for (int i = tid; i < c.r; i += kUnThreads) pos[cg + i] = c.r_pos0 + i;
       __syncthreads();
-      if (grp == 0)
-        select_lists<kUnGroup>(key, [&](int e) { return pos[e]; }, cand, mark, nE, nF, cg,
-                               fold, S, tid, gsync, [&](int i, int to) { dst[i] = to; }, [] {});
-      __syncthreads();
-      if (rank == 0 && tid == 0) {
+      auto pos_of = [&](int e) { return pos[e]; };
+      auto put = [&](int i, int to) { dst[i] = to; };
+      if (nE > 32 * kUnGroup) select_lists<kUnThreads>(key, pos_of, cand, mark, nE, nF, cg, fold, S, tid, [] { __syncthreads(); }, put, [] {});
+      else if (grp == 0) select_lists<kUnGroup>(key, pos_of, cand, mark, nE, nF, cg, fold, S, tid, gsync, put, [] {});
+      if (rank == 0 && tid == 0) {                     // (what is gathered next lies over the selection's scratch)
         L.thr[(size_t)unit * 2 + 0] = __uint_as_float(S.min_keep);
         L.thr[(size_t)unit * 2 + 1] = __uint_as_float(S.max_fold);
       }
+      __syncthreads();
     } else {
       for (int i = tid; i < c.r; i += kUnThreads) { dst[i] = c.mode == UPD_APPEND ? cg + i : -1; if (nF > 0) fold[i] = cg + i; }
       __syncthreads();
@@ -668,8 +675,7 @@ __global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int
           if (row + q * rstep < nb && jj < jn) pf[(row + q * rstep) * Y.jn + jj] = x[q];
       }
       __syncthreads();
-      // (where one group has all entries, the groups take half of the pairs each)
-      const bool halves = jn * d4 <= kUnGroup;
+      const bool halves = unit_fold_halves(Y.jn, d);   // (jn <= Y.jn)
       const int fb = halves && grp == 1 ? nb / 2 : 0, fe = halves && grp == 0 ? nb / 2 : nb;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
