@@ -262,7 +262,7 @@ struct lola_state {
   int64_t n_seen;
   int64_t launches;
   bool tensor_path = false;            // bf16, F = 64: tcgen05 kernels
-  int sms = 0;                         // SMs of the device
+  int dev = 0, sms = 0;                // the device, its SMs
   int dec_fit[9] = {};                 // generation kernel: clusters of 1 .. 8 blocks that are resident at once
   bool fused_decode = false;           // shapes the one-kernel generation step is built for
   bool have_maps = false;              // TMA descriptors of the sparse cache and the window ring exist
@@ -673,6 +673,7 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
   st->cfg = *cfg;
   st->lay = lay;
   st->base = (char*)state_dev;
+  st->dev = dev;
   st->sms = sms;
   st->n_seen = 0;
   st->launches = 0;
@@ -759,8 +760,15 @@ int lola_reset_state(lola_state* st, void* stream) {
   const StateLayout& y = st->lay;
   const ResetRanges R{y.gpos, y.gpos + U * c.sparse * 4, y.score, y.score + U * (c.sparse + c.max_chunk) * 4, y.thr, y.thr + U * 2 * 4};
   const size_t units = y.wt / 16;
-  k_reset<<<(unsigned)std::min<size_t>((units + 1023) / 1024, (size_t)st->sms * 4), 512, 0, s>>>((uint4*)st->base, units, R);
-  if (cudaGetLastError() != cudaSuccess) return LOLA_ERR_CUDA;
+  // (the caller's device need not be the state's: a fill would not mind, a kernel runs where it is launched)
+  int cur = st->dev;
+  if (cudaGetDevice(&cur) != cudaSuccess || (cur != st->dev && cudaSetDevice(st->dev) != cudaSuccess)) return LOLA_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)std::min<size_t>((units + 1023) / 1024, (size_t)st->sms * 4));
+  cfg.blockDim = dim3(512);
+  cfg.stream = s;
+  const bool ok = cudaLaunchKernelEx(&cfg, k_reset, (uint4*)st->base, units, R) == cudaSuccess;   // (its own status: not what an earlier call left)
+  if ((cur != st->dev && cudaSetDevice(cur) != cudaSuccess) || !ok) return LOLA_ERR_CUDA;
   st->n_seen = 0;
   return LOLA_OK;
 }

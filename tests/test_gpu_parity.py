@@ -414,6 +414,24 @@ def test_argument_errors_leave_state_untouched():
     ls.prefill(0, 16)                                   # the state still works
 
 
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs two devices")
+def test_reset_with_another_device_current():
+    """A layer's state is reset on the layer's device whichever one the calling thread has current, and that one stays current."""
+    from paper_2505_23666_b200 import binding
+    dev = torch.device("cuda", 1)
+    with torch.cuda.device(dev):
+        layer = binding.LolaLayer(binding.make_config(1, 2, 2, 64, 64, 16, 24, 16, dtype="f32"), torch.zeros(2, 64, 64), device=dev)
+        k = torch.randn(4, 1, 16, 2, 64, device=dev)
+        layer.prefill_chunks(None, k, k, want_out=False)
+        torch.cuda.synchronize()
+    with torch.cuda.device(0):
+        layer.reset()
+        assert torch.cuda.current_device() == 0
+    with torch.cuda.device(dev):
+        got = layer.read_state()
+    assert layer.tokens_seen == 0 and not got["window_k"].any() and not got["H"].any() and (got["sparse_pos"] == -1).all()
+
+
 def test_bounded_wait_runs_out_and_is_reported():
     """Failure path without a fault: a wait that nothing ends gives up after its limit (1 ms here) and sets
     the sticky status word; the kernels of later calls return at once, so the memories stay as they were;
