@@ -27,9 +27,10 @@ namespace lola {
 
 constexpr int kStepThreads = 256;
 constexpr int kStepQ = 8;              // query rows per unit the kernel carries
-// The stabiliser of Eq. 14 (any will do) stays 0 until a score exceeds it by this much: the blocks' sums then meet without a
-// factor, whose rounding a whole block's values would share
-constexpr float kStepLag = 64.f;
+// The stabiliser of Eq. 14 (any will do) stays 0 until a weight would exceed 2^8: most blocks' sums then meet without a factor,
+// whose rounding a whole block's values would share.  (Error of the outputs for scores below 2: 1.03e-7 - 1.06e-7 of their norm, with
+// a stabiliser that follows every score 1.05e-7 - 1.11e-7; a lag of 64 is no better, and values from 1e11 on overflowed with it.)
+constexpr float kStepLag = 5.545177f;
 
 template <int DPL>
 struct StepMsg {                       // what a block tells the others
