@@ -341,18 +341,23 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_unit_step(Layer L, Call c) 
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int i = 0; i < NC; ++i) a4[q][i] = 0.f;
+      auto add_values = [&](int but) {                 // (no pair: weight 0, values 0)
 #pragma unroll
-      for (int r0 = 0; r0 < TR; r0 += 4)               // (no pair: weight 0, values 0)
+        for (int r0 = 0; r0 < TR; r0 += 4)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float w = __shfl_sync(0xffffffffu, p, r0 + q);
+          for (int q = 0; q < 4; ++q) {
+            const float w = __shfl_sync(0xffffffffu, p, r0 + q);
+            if (r0 + q == but) continue;
 #pragma unroll
-          for (int i = 0; i < NC; i += 2) {
-            const float2 v = *reinterpret_cast<const float2*>(&X.xv[buf][r0 + q][NC * lane + i]);
-            a4[q][i] = fmaf(w, v.x, a4[q][i]);
-            a4[q][i + 1] = fmaf(w, v.y, a4[q][i + 1]);
+            for (int i = 0; i < NC; i += 2) {
+              const float2 v = *reinterpret_cast<const float2*>(&X.xv[buf][r0 + q][NC * lane + i]);
+              a4[q][i] = fmaf(w, v.x, a4[q][i]);
+              a4[q][i + 1] = fmaf(w, v.y, a4[q][i + 1]);
+            }
           }
-        }
+      };
+      if (out < 0 || whi < 0x7f800000u) add_values(-1);
+      else add_values(out);                            // its score is no number, so its value need not be finite: a weight of 0 would not keep it out
 #pragma unroll
       for (int i = 0; i < NC; ++i) {
         float y = (a4[0][i] + a4[1][i]) + (a4[2][i] + a4[3][i]);
