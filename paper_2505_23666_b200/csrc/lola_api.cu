@@ -457,9 +457,11 @@ template <int DPL>
 int launch_unit_run(lola_state* st, const Call& c, int n_chunks, bool decode, cudaStream_t s) {
   const Layer& L = st->L;
   const int K = st->unit_blocks, grid = L.B * L.Hkv * K;
-  const UnitLayout Y = unit_layout(L, K);
+  const UnitLayout Y = unit_layout(L, K, c.out ? L.g * c.nq : 0);
+  auto kernel = k_unit_run<DPL, false>;
+  if constexpr (DPL == 4) { if (Y.both) kernel = k_unit_run<DPL, true>; }
   LaunchScope scope(st, decode ? LOLA_KERNEL_DECODE : LOLA_KERNEL_RUN, s, LOLA_PATH_UNIT_RUN, grid);
-  const cudaError_t le = launch_pdl_cluster(k_unit_run<DPL>, K, dim3(grid), dim3(kUnThreads), (size_t)Y.total * 4, s, L, c, n_chunks, decode ? 1 : 0, Y);
+  const cudaError_t le = launch_pdl_cluster(kernel, K, dim3(grid), dim3(kUnThreads), (size_t)Y.total * 4, s, L, c, n_chunks, decode ? 1 : 0, Y);
   return le == cudaSuccess && cudaGetLastError() == cudaSuccess ? LOLA_OK : LOLA_ERR_CUDA;
 }
 
@@ -703,9 +705,10 @@ int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, 
     const int U = cfg->batch * cfg->n_kv_heads, smem_max = kUnSmem;
     int K = 8;
     while (K > 1 && U * K > sms) K >>= 1;
-    if (unit_layout(L, K).total * 4 <= smem_max &&
-        (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_run<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)
-                              : cudaFuncSetAttribute(k_unit_run<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) == cudaSuccess)
+    if (unit_layout_of(L, K, 0).total * 4 <= smem_max &&
+        (cfg->head_dim != 128 || cudaFuncSetAttribute(k_unit_run<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) == cudaSuccess) &&
+        (cfg->head_dim == 128 ? cudaFuncSetAttribute(k_unit_run<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)
+                              : cudaFuncSetAttribute(k_unit_run<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max)) == cudaSuccess)
       st->unit_blocks = K;
     const bool ablation = (cfg->flags & (LOLA_FLAG_QUERY_NO_LINEAR | LOLA_FLAG_QUERY_NO_SPARSE)) != 0;
     if (cfg->feat_half == 64 && cfg->sparse >= 1 && cfg->window >= 1 && L.g <= kStepQ && !ablation &&

@@ -7,8 +7,8 @@
 // memory between dependent phases and a quadratic selection.  Here a unit's H, s, W and positions stay in shared
 // memory for the whole run and the phases of a chunk are separated by cluster barriers:
 //   A  every block, two groups of 256 threads side by side:
-//        its share of E = sparse cache + leaving pairs: feature map (kept), Eq. 10 score, sent to all blocks of the cluster
-//        (prefill) its share of the queries: Eq. 14 against the H, s of the chunk's start
+//        group 0: its share of E = sparse cache + leaving pairs: feature map (kept), Eq. 10 score, sent to all blocks of the cluster
+//        group 1 (d = 128: and group 0 when it has scored): (prefill) its share of the queries: Eq. 14 against the H, s of the chunk's start
 //   -- barrier: all scores are everywhere, nobody reads the old H or ring any more
 //   B  every block for itself: the selection (Eq. 12); the feature rows of the folded pairs come from the blocks that
 //      computed them, each block folds its D / K rows of H and s (Eq. 13) and sends them to the others
@@ -16,8 +16,7 @@
 //   C  moves into the sparse cache and window roll, a warp per token
 //   -- barrier; (generation step) Eq. 14 on the updated memories
 // One group after the other a chunk took 27.0 us, side by side 22.2 (4 units of 192 pairs, 64 tokens, d = 64; 16 units of 364 pairs, two
-// heads, 93.7 and 74.4): the two share the SM's path to shared memory, which the products keep busy.  Where the scratch does not fit twice the
-// attention waits for the scores.
+// heads, 93.7 and 74.4): the two share the SM's path to shared memory, which the products keep busy.
 // K is the largest of 8, 4, 2, 1 that lets every block have an SM of its own: more blocks only shorten the phases.
 // The body of the chunk loop has to stay in the instruction cache: with everything unrolled (226 KB of code) a chunk
 // took 33 us, three quarters of it instruction fetch.  Hence short rolled loops, no integer division inside them and
@@ -39,22 +38,24 @@ constexpr int kUnRows = 32;    // members of E per scoring tile: thread = 2 rows
 constexpr int kUnQ = 8;        // query rows per batch (one per warp in the softmax)
 constexpr int kUnKeys = 256;   // keys per tile
 constexpr int kUnFold = 64;    // folded pairs per pass
-constexpr int kUnSrcFloats = 40;
+constexpr int kUnSrcFloats = 56;
 
 struct UnitLayout {            // shared memory of k_unit_run, offsets in floats
   int fp, dp;                  // F and D rounded up to a multiple of 4 (zero padding)
   int jn, jsh;                 // rows of H a block folds, and the power of two that covers them
   int phi_ld;
-  int serial;                  // the two groups share one scratch, scoring first (it does not fit twice)
+  int both;                    // group 0 attends, too, once it has scored
+  int att0;                    // from the attention scratch of group 1 to that of group 0
   int W, H, s, phi, xs, den, vf, pf, q, pq, z, p, vptr, red, row, key, pos, cand, mark, fold, dst, sel, src, part, total;
 };
 
 // Does one group of threads have all entries of a block's rows of H?  The groups then take half of the folded pairs each.
 LOLA_HD inline bool unit_fold_halves(int jn, int d) { return jn * (d / 4) <= kUnGroup; }
 
-LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
+LOLA_HD inline UnitLayout unit_layout_of(const Layer& L, int K, int both) {
+  auto imax = [](int a, int b) { return a > b ? a : b; };
   UnitLayout Y{};
-  Y.serial = serial;
+  Y.both = both;
   const int d = L.d, nE = L.lam + L.cmax, rp = (nE + K - 1) / K;
   Y.fp = (L.F + 3) & ~3;
   Y.dp = (L.D + 3) & ~3;
@@ -67,31 +68,33 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
   Y.H = take(Y.dp * d);
   Y.s = take(Y.dp);
   Y.phi = take((rp + kUnRows - 1) / kUnRows * kUnRows * Y.phi_ld);
-  // the phases of a chunk take turns in the same space
+  // the phases of a chunk take turns in the same space: first group 1's query batch beside group 0's scoring tile and then (both)
+  // query batch
   const int phase0 = o;
-  Y.xs = take(kUnRows * (d + 4));
-  Y.den = take(kUnRows);
-  int end = o;
-  if (serial) o = phase0;
   Y.q = take(kUnQ * d);
   Y.pq = take(Y.dp * kUnQ);
   Y.z = take(kUnQ * kUnKeys);              // (first the queries' u, 128 floats a row)
   Y.p = take(kUnKeys * kUnQ);
   Y.vptr = take(kUnKeys * 2);
-  Y.red = take(kUnGroup / 32 * kUnQ * 64);
   Y.row = take(kUnQ * 3);
-  end = end > o ? end : o;
+  Y.red = Y.z;                             // (after the last key tile: over z and p)
+  static_assert(kUnGroup / 32 * kUnQ * 64 <= kUnQ * kUnKeys + kUnKeys * kUnQ, "the key groups' sums do not fit");
+  Y.att0 = o - phase0;
+  int end = both ? o + Y.att0 : o;
+  Y.xs = take(kUnRows * (d + 4));
+  Y.den = take(kUnRows);
+  end = imax(end, o);
   o = phase0;
   Y.vf = take(kUnFold * d);
   Y.pf = take(kUnFold * Y.jn);
   if (unit_fold_halves(Y.jn, d)) Y.part = take(kUnGroup * 4);
-  end = end > o ? end : o;
+  end = imax(end, o);
   // the selection is over when the folded pairs come in; only its first value row is there beside it (the fold of one pair)
   o = Y.vf + d;
   Y.sel = take((int)(sizeof(SelectScratch) + 3) / 4);
   Y.cand = take(nE);
   Y.mark = take((nE + 3) / 4);
-  o = end > o ? end : o;
+  o = imax(end, o);
   Y.key = take(nE);
   Y.pos = take(nE);
   Y.fold = take(L.cmax);
@@ -101,9 +104,12 @@ LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int serial) {
   return Y;
 }
 
-LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K) {
-  const UnitLayout Y = unit_layout(L, K, 0);
-  return Y.total * 4 <= kUnSmem ? Y : unit_layout(L, K, 1);
+// rows: query rows of a unit in one chunk.  Both groups attend where a block has two batches of them or more, d = 128: with 128 registers
+// a thread one group is slower at them than 256 threads with 255 were (4 units, 200 slots, two heads, chunks of 200: one each 295 us, both
+// 226, 256 threads 289; where a block has one batch the kernel for both is 3% slower).
+LOLA_HD inline UnitLayout unit_layout(const Layer& L, int K, int rows) {
+  const UnitLayout Y = unit_layout_of(L, K, L.d == 128 && rows > K * kUnQ);
+  return Y.total * 4 <= kUnSmem ? Y : unit_layout_of(L, K, 0);
 }
 
 // Where the rows of a unit lie during one chunk (shared memory; every pointer is the unit's own first row).
@@ -112,7 +118,8 @@ struct UnitSrc {
   int cg, r_ring, ring0;         // sparse-cache members; leaving pairs that lie in the ring, and the slot of the first
   int eta, kstep;                // slots of the ring; floats between two incoming tokens
   int att_g, att_wn, att_w0;     // keys the queries see: sparse cache, window (slot of its first)
-  int tok_of[kUnQ], out_row[kUnQ];   // the query batch: token, row of q / out (-1: none)
+  int taken;                     // query batches of this block taken so far (both groups attend)
+  int tok_of[2][kUnQ], out_row[2][kUnQ];   // a group's query batch: tokens, rows of q / out (-1: none)
 };
 static_assert(sizeof(UnitSrc) <= kUnSrcFloats * 4, "UnitSrc does not fit");
 // member e of E = sparse cache ++ leaving pairs: element offset from (k ? gk : gv) etc. resolved to the row itself
@@ -209,35 +216,40 @@ __device__ __noinline__ void unit_phi(const float* u, int u_ld, float* out, int 
     for (int r = 0; r < R; ++r) ds_out[r] = ds[r];
 }
 
-// Eq. 14 for the query rows of one block of the cluster, in batches of kUnQ rows.  Key tile: a thread's whole key row
-// in two or four requests; the values (thread = 4 columns x every 16th key) are requested before the softmax.  The
-// linear term is the accumulator's first summand, with the weight of a key whose score is 0.
-template <int DPL>
-__device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const UnitLayout& Y, float* sm, UnitSrc& U, int b, int h, int rank, int K) {
+// Eq. 14 for the query rows of one block of the cluster, in batches of kUnQ rows, by group 1 or by both groups (which take the
+// batches as they get to them).  Key tile: four lanes a key; the values (thread = 4 columns x every 16th key) are requested before the
+// softmax.  The linear term is the accumulator's first summand, with the weight of a key whose score is 0.
+template <int DPL, bool BOTH>
+__device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const UnitLayout& Y, float* sm, UnitSrc& U, int b, int h, int rank, int K, int grp) {
   constexpr int d = DPL * 32, NC = d / 64, KG = kUnGroup / 16;     // NC: 64-column blocks, KG: key groups
   const int tid = threadIdx.x & (kUnGroup - 1), warp = tid >> 5, lane = tid & 31;
-  auto sync = [] { tc::named_bar_sync(2, kUnGroup); };
+  if (!BOTH) grp = 1;
+  auto sync = [grp] { tc::named_bar_sync(1 + grp, kUnGroup); };
   const int nrows = L.g * c.nq, NK = c.att_g + c.att_wn + c.att_chunk, chunk0 = c.att_g + c.att_wn;
   const float* Hs = sm + Y.H;
-  float *qs = sm + Y.q, *pq = sm + Y.pq, *zs = sm + Y.z, *ps = sm + Y.p, *red = sm + Y.red, *rw = sm + Y.row;
-  const float** vptr = reinterpret_cast<const float**>(sm + Y.vptr);
+  float* own = sm + (grp == 0 ? Y.att0 : 0);
+  float *qs = own + Y.q, *pq = own + Y.pq, *zs = own + Y.z, *ps = own + Y.p, *red = own + Y.red, *rw = own + Y.row;
+  const float** vptr = reinterpret_cast<const float**>(own + Y.vptr);
+  int *tok_of = U.tok_of[grp], *out_row = U.out_row[grp];
   const int c4 = (tid & 15) * 4, kg = tid >> 4;
 #pragma unroll 1
-  for (int row0 = rank * kUnQ; row0 < nrows; row0 += K * kUnQ) {
+  for (int row0 = rank * kUnQ; BOTH || row0 < nrows; row0 += K * kUnQ) {
+    if (BOTH && warp == 0) row0 = (rank + __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(&U.taken, 1) : 0, 0) * K) * kUnQ;
     if (tid < kUnQ) {
       const int row = row0 + tid, hl = row / c.nq, tok = row - hl * c.nq;
-      U.tok_of[tid] = tok;
-      U.out_row[tid] = row < nrows ? (b * c.nq + tok) * L.Hq + h * L.g + hl : -1;
+      tok_of[tid] = tok;
+      out_row[tid] = row < nrows ? (b * c.nq + tok) * L.Hq + h * L.g + hl : -1;
     }
     sync();
+    if (BOTH && out_row[0] < 0) break;
     if (tid < kUnQ * (d / 4)) {
-      const int rr = tid / (d / 4), row = U.out_row[rr];
+      const int rr = tid / (d / 4), row = out_row[rr];
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       if (row >= 0) x = *reinterpret_cast<const float4*>((const float*)c.q + (size_t)row * d + tid % (d / 4) * 4);
       *reinterpret_cast<float4*>(qs + tid * 4) = x;
     }
     sync();
-    // u = q W: warp = row, 4 features per lane and pass; then the feature map of two rows per warp, transposed into pq
+    // u = q W: warp = row, 4 features per lane and pass; then the row's feature map, transposed into pq
     const bool two = Y.fp <= 64;                       // (half a warp has all features: the other half takes half of the inner dimension)
 #pragma unroll 1
     for (int f = (two ? lane & 15 : lane) * 4; f < Y.fp; f += 128) {
@@ -335,7 +347,7 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
             const float keep = sub & 1 ? z[p][r + 2] : z[p][r], give = sub & 1 ? z[p][r] : z[p][r + 2];
             const float zz = keep + __shfl_xor_sync(0xffffffffu, give, 1);
             const int row = (sub & 2) * 2 + (sub & 1) * 2 + r;
-            zs[row * kUnKeys + kb] = kb < nk && (ci < 0 || ci <= U.tok_of[row]) ? zz * L.scale : -CUDART_INF_F;
+            zs[row * kUnKeys + kb] = kb < nk && (ci < 0 || ci <= tok_of[row]) ? zz * L.scale : -CUDART_INF_F;
           }
         }
       }
@@ -404,14 +416,15 @@ __device__ __forceinline__ void unit_attend(const Layer& L, const Call& c, const
         float a = 0.f;
 #pragma unroll
         for (int w = 0; w < kUnGroup / 32; ++w) a += red[(w * kUnQ + r) * 64 + cc];
-        if (U.out_row[r] >= 0) ((float*)c.out)[(size_t)U.out_row[r] * d + nc * 64 + cc] = a / rw[kUnQ + r];
+        if (out_row[r] >= 0) ((float*)c.out)[(size_t)out_row[r] * d + nc * 64 + cc] = a / rw[kUnQ + r];
       }
       sync();
     }
   }
 }
 
-template <int DPL>
+// BOTH: group 0 attends, too
+template <int DPL, bool BOTH>
 __global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int n_chunks, int decode, UnitLayout Y) {
   namespace co = cooperative_groups;
   constexpr int d = DPL * 32, d4 = d / 4;
@@ -476,6 +489,7 @@ __global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int
       U.att_g = c.att_g;
       U.att_wn = c.att_wn;
       U.att_w0 = L.eta > 0 ? c.att_w0 % L.eta : 0;
+      if (BOTH) U.taken = 0;
     }
     __syncthreads();
     // ---- A: feature rows and scores of this block's members of E
@@ -565,13 +579,13 @@ __global__ void __launch_bounds__(kUnThreads, 1) k_unit_run(Layer L, Call c, int
       }
       gsync();
     }
-    if (Y.serial && ne > 0 && c.out && (!decode || it == 1)) __syncthreads();
-    if (grp == 1 && c.out && (!decode || it == 1)) unit_attend<DPL>(L, c, Y, sm, U, b, h, rank, K);
+    if ((BOTH || grp == 1) && c.out && (!decode || it == 1)) unit_attend<DPL, BOTH>(L, c, Y, sm, U, b, h, rank, K, grp);
     if (decode && it == 1) break;
     cl.sync();
     // ---- B: which pairs fold, which leaving pairs stay
     // One leaving pair, one fold (a generation step on full caches): the lowest score is all there is to find, and every
-    // block folds that pair into its whole copy of H (31 -> 26 us a step: no lists, and no exchange of rows of H)
+    // block folds that pair into its whole copy of H: no lists, and no exchange of rows of H (F = 32, 4 units: 23.6 us a step, with lists
+    // 26.5; 80 units 47.5 and 50.6)
     const bool one = scored && nF == 1 && c.r == 1;
     if (one) {
       if (tid == 0) pos[cg] = c.r_pos0;
