@@ -274,7 +274,8 @@ enum {
   LOLA_PATH_DECODE_FUSED_LONG = 1u << 10,/* (never reported: LOLA_PATH_DECODE_FUSED serves every length)      */
   LOLA_PATH_H_IMAGE_REBUILD = 1u << 11,  /* (never reported: every kernel reads H itself)                   */
   LOLA_PATH_UNIT_RUN = 1u << 12,         /* fp32: a run of chunks, or a generation step, as one kernel      */
-  LOLA_PATH_PREFILL_RUN = 1u << 13       /* bf16: a run of chunks as one kernel                             */
+  LOLA_PATH_PREFILL_RUN = 1u << 13,      /* bf16: a run of chunks as one kernel                             */
+  LOLA_PATH_UNIT_STEP = 1u << 14         /* beside LOLA_PATH_UNIT_RUN: a generation step of the kernel for F = 64 */
 };
 typedef struct lola_call_info {
   uint32_t paths;                        /* OR of LOLA_PATH_*                                               */

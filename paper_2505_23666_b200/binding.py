@@ -44,7 +44,7 @@ class lola_call_info(C.Structure):
 
 PATH_BITS = ["attend_tma", "attend_mma", "attend_generic", "score_tma", "score_mma", "score_generic", "select_kernel",
              "apply_tma", "update_generic", "decode_fused", "decode_fused_long", "h_image_rebuild",
-             "unit_run", "prefill_run"]
+             "unit_run", "prefill_run", "unit_step"]
 LOLA_STATUS_SELFTEST = 128
 LOLA_FLAG_GENERIC_KERNELS, LOLA_FLAG_QUERY_NO_LINEAR, LOLA_FLAG_QUERY_NO_SPARSE = 1, 4, 8
 
