@@ -84,7 +84,8 @@ typedef struct lola_config {
   int32_t dtype;         /* lola_dtype of q, k, v, out, W and of the cached keys/values.
                             H, s, scores and all softmax statistics are always fp32.
                             LOLA_BF16 additionally rounds phi(K) and H to bf16 inside the Eq. 10
-                            contraction and folds the rounded phi(K) (Eq. 13).                  */
+                            contraction; Eq. 13 folds phi(K) in two or three bf16 parts, or (generation
+                            steps on full caches of whole 64-slot blocks) rounded to bf16.       */
   int32_t phi_kind;      /* lola_phi                                                            */
   float softmax_scale;   /* 0 => 1/sqrt(head_dim) (Eq. 2)                                       */
   uint32_t flags;        /* 0, or an OR of LOLA_FLAG_*                                          */
@@ -117,8 +118,8 @@ typedef struct lola_state_view {
 
 /* Device bytes the caller must provide for one state (a multiple of 256).  0 if cfg is invalid.
  * Holds H, s, the sparse cache with positions and scores, the window ring, for bf16 layers with
- * feat_half = 64 the tensor-core operand images of W (per KV head) and of H (per unit), and the small per-unit
- * work lists the update kernels pass to each other.                                             */
+ * feat_half = 64 the tensor-core operand image of W (per KV head), and the small per-unit work lists the update
+ * kernels pass to each other.                                                                   */
 size_t lola_state_bytes(const lola_config* cfg);
 
 /* Pseudo-code `init`: empty window, empty sparse cache, H = 0, s = 0.
@@ -131,7 +132,8 @@ size_t lola_state_bytes(const lola_config* cfg);
 int lola_init_state(const lola_config* cfg, const void* W_dev, void* state_dev, size_t state_bytes,
                     void* stream, lola_state** out);
 
-/* Back to the state lola_init_state leaves (pseudo-code `init`), asynchronously on `stream`. */
+/* Back to the state lola_init_state leaves (pseudo-code `init`), asynchronously on `stream` (of the state's device, whichever
+ * device the caller has current). */
 int lola_reset_state(lola_state* st, void* stream);
 
 /* Chunkwise inference (section "Chunkwise Inference", Eq. 15): attend, then evict.
