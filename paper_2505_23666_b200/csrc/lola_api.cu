@@ -508,15 +508,15 @@ int launch_prefill_run(lola_state* st, const Call& c, int n_chunks, cudaStream_t
 }
 
 // Attention and scoring blocks per unit (A, N) of the prefill kernel that has both, for chunks of n tokens on full caches; A = 0
-// where its clusters do not fit or the three-kernel chain is faster.  Microseconds of the parts, measured at d = 128: an
-// item (two query tiles) 6 + 2.1 per key tile, 8 around them; scoring 4.8 per pair of tiles and block, selection and fold
-// 11 and 4 per further 64 pairs (16 units, chunks of 256: 34.9 a chunk; counted as 3, 24 units with chunks of
-// 96 took 28.4, now 24.6, 8 units of 100, d = 64, 23.9, now 20.3).  The chain: an attention block (an item) 7 + 2.1 per key tile, in rounds of the SMs; 2.6 per
-// scored tile on the SMs it leaves; 10 and 11 per further 64 pairs for the fold.  (64 units, 8 heads: chunks of 64 tokens
-// 53 here, 56 there; chunks of 256: 198 here, 147 there.)  The set-up of a run, 6, is shared by its chunks (64 units, 4 heads:
-// 36 a chunk alone, 29 in a run; 34.5 there).  With d = 64 both sides are shorter, and the same choices are the faster ones:
-// 64 units with 2, 4, 8 heads 18.5, 21.8, 36.3 here, 23.6, 26.7, 37.1 there; 24 units, 8 heads, chunks of 40 18.7 and 23.8; 32
-// units, 8 heads, lambda 960 24.7 and 28.0; 16 units, chunks of 256 30.4 and 41.9.
+// where its clusters do not fit or the three-kernel chain is faster.  Microseconds of the parts at d = 128, from when the selection took
+// 7 us (it takes 4 now, in both): an item (two query tiles) 6 + 2.1 per key tile, 8 around them; scoring 4.8 per pair of tiles and block,
+// selection and fold 11 and 4 per further 64 pairs.  The chain: an attention block (an item) 7 + 2.1 per key tile, in rounds of
+// the SMs; 2.6 per scored tile on the SMs it leaves; 10 and 11 per further 64 pairs for the fold.  The set-up of a run, 6, is shared by its
+// chunks.  The choices, measured with what the kernels take now (a chunk of a run of 16, here and there; d = 128, then d = 64): 64 units
+// of 832 slots, 4 heads 30 and 37, 27 and 31, 8 heads 53.4 and 53.2, 49 and 47; 48 of 500, 8 heads 42 and 33, 38 and 29; chunks of 256, 16 units of
+// 512, 4 heads 35 and 61, 30 and 47, 64 units 121 and 102, 105 and 83; of 128, 32 units of 960, 4 heads 38 and 52, 34 and 42; of 96, 24 units of
+// 500, 4 heads 28 and 41, 25 and 34.  Of 60 shapes it takes the slower one for four, all of 8 heads: by 4% (64 units of 832, d = 64, and 32 of
+// 960, chunks of 128) to 8% (the latter with d = 64, and 16 of 512, chunks of 256); and for single chunks of 64 units with 8 heads (65 and 56).
 struct TeamShape { int A, N; };
 inline TeamShape team_shape(const lola_state* st, int n, int n_chunks) {
   const Layer& L = st->L;
